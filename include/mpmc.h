@@ -244,9 +244,15 @@ int mpmc_rhs_adjoint(mpmc_ctx* ctx, const double* U, const mpmc_stage* stage, co
  * and U^(2), which spare the reverse step their recomputation. */
 int mpmc_rk_step_record(mpmc_ctx* ctx, double* U, double dt, uint32_t* tape, double* U_stages, double* W_stages);
 
+/* One SSP-RK3 step in place in the arithmetic of mpmc_rk_step_record (bit for
+ * bit the states that it records; mpmc_rk_step and mpmc_step_n round
+ * otherwise): the forward step of a differentiated run.  dt as for
+ * mpmc_rk_step; dt_out (nullable, device double) receives the step's length. */
+int mpmc_rk_step_replay(mpmc_ctx* ctx, double* U, double dt, double* dt_out);
+
 /* Reverse of one SSP-RK3 step (Eq. SSPRK3) from U_n:
  *   lam_n = (dU^{n+1}/dU^n)^T lam_next.
- * dt: as passed to mpmc_rk_step (<= 0: the CFL step of U_n, recomputed
+ * dt: as passed to mpmc_rk_step_record (<= 0: the CFL step of U_n, recomputed
  * bit-identically).  U_stages (nullable): the step's stage states from
  * mpmc_rk_step_record; recomputed from U_n when null.  W_stages (nullable;
  * only with U_stages): that call's primitive caches, used instead of

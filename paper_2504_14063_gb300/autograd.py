@@ -44,7 +44,7 @@ class _RKStep(torch.autograd.Function):
     def forward(fctx, ctx, U, dt):
         U = U.detach().contiguous()
         out = U.clone()
-        ctx.rk_step(out, dt)
+        ctx.rk_step_replay(out, dt)
         fctx.ctx = ctx
         fctx.dt = dt
         fctx.save_for_backward(U)
@@ -97,12 +97,9 @@ class _Rollout(torch.autograd.Function):
         for k in range(n):
             if k % every == 0:
                 ckpts.append(U.clone())
-            if dt > 0.0:
-                ctx.rk_step(U, dt)              # fixed step
-                dts[k] = dt
-            else:
-                ctx.step_n(U, 1, slot)          # CFL step of U^k, recorded
-                dts[k] = slot[0]
+            # a step of fixed length, or the CFL step of U^k, recorded
+            ctx.rk_step_replay(U, dt, slot)
+            dts[k] = slot[0]
             if probe is not None:
                 J += dts[k] * _probe_term(ctx, U, probe)
         fctx.ctx, fctx.n, fctx.every, fctx.probe = ctx, n, every, probe

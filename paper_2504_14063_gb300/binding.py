@@ -79,6 +79,7 @@ def _load():
         "mpmc_dt_gamma": (i, [vp, vp, vp]),
         "mpmc_rhs_adjoint": (i, [vp, vp, ctypes.POINTER(StageC), vp, vp, vp]),
         "mpmc_rk_step_record": (i, [vp, vp, d, vp, vp, vp]),
+        "mpmc_rk_step_replay": (i, [vp, vp, d, vp]),
         "mpmc_rk_step_adjoint": (i, [vp, vp, vp, vp, d, vp, vp, vp]),
         "mpmc_init_state_adjoint": (i, [vp, vp, vp, vp]),
         "mpmc_primitives": (i, [vp, vp, vp]),
@@ -280,6 +281,12 @@ class Context:
         self._check(lib.mpmc_rk_step_record(self.h, _dev(U), float(dt), _ptr(tape), _dev(stages),
                                             self._wstages(wstages)))
         return stages
+
+    def rk_step_replay(self, U, dt=0.0, dt_out=None):
+        """One SSP-RK3 step in place, bit for bit the one rk_step_record takes;
+        dt_out (1 double, device) receives its length."""
+        self._check(lib.mpmc_rk_step_replay(self.h, _dev(U), float(dt), _ptr(dt_out)))
+        return U
 
     def rk_step_adjoint(self, U_n, lam_next, dt=0.0, tape=None, lam_n=None, stages=None, wstages=None):
         """lam_n = (dU^{n+1}/dU^n)^T lam_next for the SSP-RK3 step from U_n

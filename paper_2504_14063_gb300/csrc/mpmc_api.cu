@@ -20,6 +20,7 @@ static constexpr int NFAM_MAX = 6;
 struct mpmc_ctx {
   KParams P;
   Ops ops;
+  Ops rec;   // the recording calls' kernels (FP64: plain FP64 arithmetic; else ops)
   AdjOps aops;
   int precision;
   cudaStream_t stream;
@@ -214,7 +215,16 @@ extern "C" int mpmc_create(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_m
     c->ops.face = mixed ? face_mixed_teno6(D, ns) : face_fp64_teno6(D, ns);
     c->aops.face = adj_face_teno6(D, ns);
   }
-  if (!c->ops.face || !c->aops.face) {
+  c->rec = c->ops;
+  if (!mixed) {
+    switch (P.recon) {
+      case MPMC_RECON_WENO5JS: c->ops.face = face_fast_weno5js(D, ns); break;
+      case MPMC_RECON_TENO5: c->ops.face = face_fast_teno5(D, ns); break;
+      case MPMC_RECON_TENO6: c->ops.face = face_fast_teno6(D, ns); break;
+      default: c->ops.face = face_fast_weno5z(D, ns); break;
+    }
+  }
+  if (!c->ops.face || !c->rec.face || !c->aops.face) {
     delete c;
     return MPMC_INVALID_ARG;
   }
@@ -319,48 +329,47 @@ extern "C" int mpmc_init_state(mpmc_ctx* c, const double* prim, double* U) {
 // ---------------------------------------------------------------------------
 // one stage: faces of every direction from the primitive cache of Uk, then
 // the fused divergence / RK combination
-static void stage(mpmc_ctx* c, cudaStream_t s, const double* Un, const double* Uk, double rk0, double rk1, double rk2,
-                  double* Uout, double* dUdt, uint32_t* flags) {
+static void stage(mpmc_ctx* c, const Ops& ops, cudaStream_t s, const double* Un, const double* Uk, double rk0,
+                  double rk1, double rk2, double* Uout, double* dUdt, uint32_t* flags) {
   const KParams& P = c->P;
   long long off = 0;
   const double* Gk = Uk == Un ? c->Uin : c->Gk;   // the ghost buffer of U^(k)
   for (int d = 0; d < P.dim; ++d) {
     ProfScope ps(c, FAM_FACE, s);
-    c->ops.face(P, s, d, c->Wc, Un, Uk, Gk, c->scal, rk0, rk1, rk2, c->F[d], flags ? flags + off : nullptr,
-                c->stats);
+    ops.face(P, s, d, c->Wc, Un, Uk, Gk, c->scal, rk0, rk1, rk2, c->F[d], flags ? flags + off : nullptr, c->stats);
     off += c->nface[d];
   }
   ProfScope ps(c, FAM_UPDATE, s);
-  c->ops.update(P, s, Un, Uk, c->F, c->scal, rk0, rk1, rk2, Uout, dUdt, c->status);
+  ops.update(P, s, Un, Uk, c->F, c->scal, rk0, rk1, rk2, Uout, dUdt, c->status);
 }
 
 // primitive cache of U; the pass that computes dt and Gamma (red != null)
 // is the one of U^n, every other one of a stage state: each first fills its
 // ghost buffer's characteristic ghosts
-static void prim(mpmc_ctx* c, cudaStream_t s, const double* U, unsigned long long* red) {
+static void prim(mpmc_ctx* c, const Ops& ops, cudaStream_t s, const double* U, unsigned long long* red) {
   ProfScope ps(c, FAM_PRIM, s);
   double* G = red ? c->Uin : c->Gk;
-  if (c->P.nslots) c->ops.ghost(c->P, s, U, G);
-  c->ops.prim(c->P, s, U, G, c->Wc, red, c->status);
+  if (c->P.nslots) ops.ghost(c->P, s, U, G);
+  ops.prim(c->P, s, U, G, c->Wc, red, c->status);
 }
 
 // dt and Gamma from U (prim pass with the block maxima), then k_dt
-static void dt_gamma(mpmc_ctx* c, cudaStream_t s, const double* U, double dt_fixed, double gamma_fixed,
-                     double* hist) {
-  prim(c, s, U, c->red);
+static void dt_gamma(mpmc_ctx* c, const Ops& ops, cudaStream_t s, const double* U, double dt_fixed,
+                     double gamma_fixed, double* hist) {
+  prim(c, ops, s, U, c->red);
   ProfScope ps(c, FAM_DT, s);
   k_dt<<<1, 1, 0, s>>>(c->P, c->red, c->scal, dt_fixed, gamma_fixed, hist, c->counter);
 }
 
 // Eq. SSPRK3 with U^n = U, result written back to U
-static void rk3(mpmc_ctx* c, cudaStream_t s, double* U, double dt, uint32_t* tape, double* hist) {
-  dt_gamma(c, s, U, dt, -1.0, hist);
+static void rk3(mpmc_ctx* c, const Ops& ops, cudaStream_t s, double* U, double dt, uint32_t* tape, double* hist) {
+  dt_gamma(c, ops, s, U, dt, -1.0, hist);
   const long long nf = c->nface_total;
-  stage(c, s, U, U, 1.0, 0.0, 1.0, c->U1, nullptr, tape);
-  prim(c, s, c->U1, nullptr);
-  stage(c, s, U, c->U1, 0.75, 0.25, 0.25, c->U2, nullptr, tape ? tape + nf : nullptr);
-  prim(c, s, c->U2, nullptr);
-  stage(c, s, U, c->U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, U, nullptr, tape ? tape + 2 * nf : nullptr);
+  stage(c, ops, s, U, U, 1.0, 0.0, 1.0, c->U1, nullptr, tape);
+  prim(c, ops, s, c->U1, nullptr);
+  stage(c, ops, s, U, c->U1, 0.75, 0.25, 0.25, c->U2, nullptr, tape ? tape + nf : nullptr);
+  prim(c, ops, s, c->U2, nullptr);
+  stage(c, ops, s, U, c->U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, U, nullptr, tape ? tape + 2 * nf : nullptr);
 }
 
 extern "C" int mpmc_rhs(mpmc_ctx* c, const double* U, double* dUdt, const mpmc_stage* st, uint32_t* flags) {
@@ -371,16 +380,16 @@ extern "C" int mpmc_rhs(mpmc_ctx* c, const double* U, double* dUdt, const mpmc_s
   cudaStream_t s = c->stream;
   // dt / Gamma from U^n (always run so that the prim pass of U_n also
   // validates it); then the primitive cache of U
-  dt_gamma(c, s, Un, dt, G, nullptr);
-  if (Un != U) prim(c, s, U, nullptr);
-  stage(c, s, Un, U, rk0, rk1, rk2, nullptr, dUdt, flags);
+  dt_gamma(c, c->ops, s, Un, dt, G, nullptr);
+  if (Un != U) prim(c, c->ops, s, U, nullptr);
+  stage(c, c->ops, s, Un, U, rk0, rk1, rk2, nullptr, dUdt, flags);
   c->faces_done += c->nface_total;
   return check_launch(c, "rhs");
 }
 
 extern "C" int mpmc_rk_step(mpmc_ctx* c, double* U, double dt, uint32_t* tape) {
   if (!c || !U) return fail(c, MPMC_INVALID_ARG, "rk_step: null argument");
-  rk3(c, c->stream, U, dt, tape, nullptr);
+  rk3(c, c->ops, c->stream, U, dt, tape, nullptr);
   c->faces_done += 3ull * c->nface_total;
   return check_launch(c, "rk_step");
 }
@@ -400,7 +409,7 @@ extern "C" int mpmc_step_n(mpmc_ctx* c, double* U, int n, double t_end, double* 
     if (cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
       return fail(c, MPMC_CUDA_ERROR, "step_n: capture begin failed");
     c->capturing = true;
-    rk3(c, c->cap, U, 0.0, nullptr, dt_out);
+    rk3(c, c->ops, c->cap, U, 0.0, nullptr, dt_out);
     c->capturing = false;
     if (cudaStreamEndCapture(c->cap, &graph) != cudaSuccess) {
       cudaGetLastError();
@@ -446,7 +455,7 @@ extern "C" int mpmc_step_n_host(mpmc_ctx* c, double* U_host, int n) {
 
 extern "C" int mpmc_dt_gamma(mpmc_ctx* c, const double* U, double* out_dev) {
   if (!c || !U || !out_dev) return fail(c, MPMC_INVALID_ARG, "dt_gamma: null argument");
-  dt_gamma(c, c->stream, U, 0.0, -1.0, nullptr);
+  dt_gamma(c, c->ops, c->stream, U, 0.0, -1.0, nullptr);
   cudaMemcpyAsync(out_dev, c->scal, 2 * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
   return check_launch(c, "dt_gamma");
 }
@@ -477,7 +486,7 @@ static void faces_only(mpmc_ctx* c, cudaStream_t s, const double* Un, const doub
   const double* Gk = Uk == Un ? c->Uin : c->Gk;
   for (int d = 0; d < c->P.dim; ++d) {
     ProfScope ps(c, FAM_FACE, s);
-    c->ops.face(c->P, s, d, c->Wc, Un, Uk, Gk, c->scal, rk0, rk1, rk2, c->F[d], flags + off, nullptr);
+    c->rec.face(c->P, s, d, c->Wc, Un, Uk, Gk, c->scal, rk0, rk1, rk2, c->F[d], flags + off, nullptr);
     off += c->nface[d];
   }
 }
@@ -514,14 +523,23 @@ extern "C" int mpmc_rhs_adjoint(mpmc_ctx* c, const double* U, const mpmc_stage* 
   const double dt = st ? st->dt : 0.0, G = st ? st->Gamma : -1.0;
   cudaStream_t s = c->stream;
   // the same dt / Gamma and primitive cache as mpmc_rhs
-  dt_gamma(c, s, Un, dt, G, nullptr);
-  if (Un != U) prim(c, s, U, nullptr);
+  dt_gamma(c, c->rec, s, Un, dt, G, nullptr);
+  if (Un != U) prim(c, c->rec, s, U, nullptr);
   if (!tape) {
     faces_only(c, s, Un, U, rk0, rk1, rk2, c->tape_int);
     tape = c->tape_int;
   }
   stage_vjp(c, s, U, (const double*)c->Wc, tape, lam_dUdt, 1.0, 0, lam_U, 1.0, lam_U, 0.0, nullptr, 0.0, nullptr);
   return check_launch(c, "rhs_adjoint");
+}
+
+extern "C" int mpmc_rk_step_replay(mpmc_ctx* c, double* U, double dt, double* dt_out) {
+  if (!c || !U) return fail(c, MPMC_INVALID_ARG, "rk_step_replay: null argument");
+  cudaStream_t s = c->stream;
+  if (dt_out) cudaMemsetAsync(c->counter, 0, sizeof(int), s);
+  rk3(c, c->rec, s, U, dt, nullptr, dt_out);
+  c->faces_done += 3ull * c->nface_total;
+  return check_launch(c, "rk_step_replay");
 }
 
 extern "C" int mpmc_rk_step_record(mpmc_ctx* c, double* U, double dt, uint32_t* tape, double* U_stages,
@@ -540,15 +558,15 @@ extern "C" int mpmc_rk_step_record(mpmc_ctx* c, double* U, double dt, uint32_t* 
     return !W_stages || cudaMemcpyAsync(W_stages + k * nw, c->Wc, nw * sizeof(double), cudaMemcpyDeviceToDevice,
                                         s) == cudaSuccess;
   };
-  dt_gamma(c, s, U, dt, -1.0, nullptr);
+  dt_gamma(c, c->rec, s, U, dt, -1.0, nullptr);
   if (!keep(0)) return fail(c, MPMC_CUDA_ERROR, "rk_step_record: cache copy");
-  stage(c, s, U, U, 1.0, 0.0, 1.0, U1, nullptr, tape);
-  prim(c, s, U1, nullptr);
+  stage(c, c->rec, s, U, U, 1.0, 0.0, 1.0, U1, nullptr, tape);
+  prim(c, c->rec, s, U1, nullptr);
   if (!keep(1)) return fail(c, MPMC_CUDA_ERROR, "rk_step_record: cache copy");
-  stage(c, s, U, U1, 0.75, 0.25, 0.25, U2, nullptr, tape ? tape + nf : nullptr);
-  prim(c, s, U2, nullptr);
+  stage(c, c->rec, s, U, U1, 0.75, 0.25, 0.25, U2, nullptr, tape ? tape + nf : nullptr);
+  prim(c, c->rec, s, U2, nullptr);
   if (!keep(2)) return fail(c, MPMC_CUDA_ERROR, "rk_step_record: cache copy");
-  stage(c, s, U, U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, U, nullptr, tape ? tape + 2 * nf : nullptr);
+  stage(c, c->rec, s, U, U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, U, nullptr, tape ? tape + 2 * nf : nullptr);
   c->faces_done += 3ull * c->nface_total;
   return check_launch(c, "rk_step_record");
 }
@@ -562,26 +580,26 @@ extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double
   const KParams& P = c->P;
   const long long nf = c->nface_total, n = (long long)P.nv * P.ncell;
   cudaStream_t s = c->stream;
-  dt_gamma(c, s, U_n, dt, -1.0, nullptr);
+  dt_gamma(c, c->rec, s, U_n, dt, -1.0, nullptr);
   const double* U1 = U_stages ? U_stages : c->U1;
   const double* U2 = U_stages ? U_stages + n : c->U2;
   uint32_t* tp = tape ? nullptr : c->tape_int;
   if (!U_stages) {
     // forward recomputation of the stage states (and of the flags if no tape)
-    stage(c, s, U_n, U_n, 1.0, 0.0, 1.0, c->U1, nullptr, tp);
-    prim(c, s, c->U1, nullptr);
-    stage(c, s, U_n, c->U1, 0.75, 0.25, 0.25, c->U2, nullptr, tp ? tp + nf : nullptr);
-    prim(c, s, c->U2, nullptr);
+    stage(c, c->rec, s, U_n, U_n, 1.0, 0.0, 1.0, c->U1, nullptr, tp);
+    prim(c, c->rec, s, c->U1, nullptr);
+    stage(c, c->rec, s, U_n, c->U1, 0.75, 0.25, 0.25, c->U2, nullptr, tp ? tp + nf : nullptr);
+    prim(c, c->rec, s, c->U2, nullptr);
     if (tp) faces_only(c, s, U_n, c->U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, tp + 2 * nf);
   } else if (tp) {
     // stage states given, flags recomputed
     faces_only(c, s, U_n, U_n, 1.0, 0.0, 1.0, tp);
-    prim(c, s, U1, nullptr);
+    prim(c, c->rec, s, U1, nullptr);
     faces_only(c, s, U_n, U1, 0.75, 0.25, 0.25, tp + nf);
-    prim(c, s, U2, nullptr);
+    prim(c, c->rec, s, U2, nullptr);
     faces_only(c, s, U_n, U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, tp + 2 * nf);
   } else if (!W_stages) {
-    prim(c, s, U2, nullptr);
+    prim(c, c->rec, s, U2, nullptr);
   }
   const uint32_t* T = tape ? tape : c->tape_int;
   // the primitive cache of each stage state: kept by mpmc_rk_step_record, or
@@ -596,10 +614,10 @@ extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double
   double* l1 = c->lamA;
   stage_vjp(c, s, U2, W_stages ? W_stages + 2 * nw : Wc, T + 2 * nf, lam_next, 2.0 / 3.0, 1, l2, 2.0 / 3.0,
             lam_next, 0.0, nullptr, 0.0, nullptr);
-  if (!W_stages) prim(c, s, U1, nullptr);
+  if (!W_stages) prim(c, c->rec, s, U1, nullptr);
   stage_vjp(c, s, U1, W_stages ? W_stages + nw : Wc, T + nf, l2, 0.25, 1, l1, 0.25, l2, 0.0, nullptr, 0.0,
             nullptr);
-  if (!W_stages) prim(c, s, U_n, nullptr);
+  if (!W_stages) prim(c, c->rec, s, U_n, nullptr);
   stage_vjp(c, s, U_n, W_stages ? W_stages : Wc, T, l1, 1.0, 1, lam_n, 1.0 / 3.0, lam_next, 0.75, l2, 1.0, l1);
   return check_launch(c, "rk_step_adjoint");
 }
@@ -616,7 +634,7 @@ extern "C" int mpmc_primitives(mpmc_ctx* c, const double* U, double* out) {
   if (!c || !U || !out) return fail(c, MPMC_INVALID_ARG, "primitives: null argument");
   if (c->precision != MPMC_FP64) return fail(c, MPMC_INVALID_ARG, "primitives: needs an FP64 context");
   const KParams& P = c->P;
-  prim(c, c->stream, U, nullptr);
+  prim(c, c->rec, c->stream, U, nullptr);
   if (cudaMemcpy2DAsync(out, (size_t)P.ncell * sizeof(double), c->Wc, (size_t)P.wstride * sizeof(double),
                         (size_t)P.ncell * sizeof(double), (size_t)nprim_fields(P), cudaMemcpyDeviceToDevice,
                         c->stream) != cudaSuccess)

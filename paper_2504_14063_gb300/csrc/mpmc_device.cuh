@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "mpmc_ff.h"
 #include "mpmc_narrow.h"
 
 namespace mpmc {
@@ -71,6 +72,8 @@ struct KParams {
     float W[MAXS], mu[MAXS], Sc[MAXS], wilke[MAXS][MAXS];
     float inv_dx, cdi_eps, sharp0, mu_liquid, prandtl, lambda_liquid;
   } f32;
+  // read by the forward FP64 passes (mpmc_fast.cuh)
+  WenoEps weno_eps4;  // 4 weno_eps, for the float-float WENO5-Z
 };
 
 // fills P.f32 from the FP64 fields (host)

@@ -1,0 +1,472 @@
+// The forward FP64 face pass (arXiv 2504.14063): mpmc_kernels.cuh's k_face
+// with the parts of its arithmetic that act on the cells' differences only
+// moved from the FP64 pipe (2 operations per clock and SM on GB300) to
+// float-float on the FP32 pipe (mpmc_ff.h says what that rests on).  The
+// FP64 pipe bounds the pass (86 % busy); WENO5-Z was half of its operations.
+// Face passes of one SSP-RK3 step with all interpolation in FP64 and so:
+// shock-bubble 1024 x 512 8.70 -> 5.44 ms, droplet field 128^3 79.7 -> 54.2 ms.
+// The right-hand sides' error against extended precision went from 1 to
+// 0.5 .. 1.1 of the FP64 form's (four workloads, every field).
+//
+// Steps and right-hand sides run these kernels.  The recording calls of the
+// discrete adjoint (mpmc_rk_step_record and what mpmc_rk_step_adjoint and
+// mpmc_rhs_adjoint recompute) run mpmc_kernels.cuh's: the reverse sweep
+// evaluates the faces in that form, and the derivative it takes is
+// discontinuous in the states' rounding (the mass-fraction limiter acts
+// unless sum Y is one to 1e-15, a stencil of rounding noise has weights of
+// its own), so the states it linearizes at keep that form's rounding.
+#pragma once
+#include "mpmc_kernels.cuh"
+
+namespace mpmc {
+namespace fast {
+
+// the FP64 form of both sides, for stencils outside the range of the
+// float-float one (differences that are not finite or beyond 2^900); out of
+// line, so that it costs the callers no registers
+static __device__ __noinline__ double2 weno5z_lr_fp64(double w0, double w1, double w2, double w3, double w4,
+                                                      double w5, double eps) {
+  const double w[6] = {w0, w1, w2, w3, w4, w5};
+  double L, R;
+  mpmc::recon_lr<RC_WENO5Z>(w, eps, L, R);
+  return make_double2(L, R);
+}
+
+// both face values of one field from the cells y[0..5] = i-2..i+3 around
+// the face i+1/2; WENO5-Z in float-float (mpmc_ff.h)
+template <int RC>
+__device__ __forceinline__ void recon_lr(const KParams& P, const double* y, double& L, double& R) {
+  if constexpr (RC == RC_WENO5Z) {
+    if (!weno5z_lr_ff(y, P.weno_eps4, L, R)) {
+      const double2 v = weno5z_lr_fp64(y[0], y[1], y[2], y[3], y[4], y[5], P.weno_eps);
+      L = v.x;
+      R = v.y;
+    }
+  } else {
+    mpmc::recon_lr<RC>(y, P.weno_eps, L, R);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// DIR: the face direction, a template parameter so that every array indexed
+// by it is indexed by a constant (registers, not the stack).  RC: the
+// ENO-type interpolation (RC_WENO5Z, the method's, or one of Sec. 4.1's others)
+template <int NS, int D, int DIR, int RC>
+__global__ void __launch_bounds__(FACE_THREADS)
+    k_face(const KParams P, const double* __restrict__ Wc, const double* __restrict__ Un,
+           const double* __restrict__ Uk, const double* __restrict__ Uin, const double* __restrict__ scal,
+           const double rk0, const double rk1, const double rk2, double* __restrict__ F,
+           uint32_t* __restrict__ flags, unsigned long long* __restrict__ stats) {
+  constexpr int NV = NS + D + 1;
+  constexpr int d = DIR;
+  const int f0 = P.n[0] + (d == 0), f1 = P.n[1] + (d == 1), f2 = P.n[2] + (d == 2);
+  const long long nf = (long long)f0 * f1 * f2;
+  const long long fid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (fid >= nf) return;
+  int fc[3];
+  unflatten(fid, f0, f1, fc);
+  int ci[3] = {fc[0], fc[1], fc[2]};
+  ci[d] -= 1;  // the cell on the low side of the face
+  const double dt = scal[0], Gamma = scal[1];
+  const long long ws = P.wstride;
+
+  CRef cr[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    int cc[3] = {ci[0], ci[1], ci[2]};
+    cc[d] += j - 2;
+    cr[j] = map_cell_m<1u << d>(P, cc[0], cc[1], cc[2]);
+  }
+  const CRef ri = cr[2], rj = cr[3];
+  uint32_t fl = 0u;
+
+  // step 1: averaged conserved state on the face, its EOS, the scalars of
+  // the characteristic matrices (Appendix A)
+  double X, c, ic;
+  {
+    double Ui[NV], Uj[NV];
+    load_U<NS, D>(P, Uk, Uin, ri, Ui);
+    load_U<NS, D>(P, Uk, Uin, rj, Uj);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Ui[v] = 0.5 * (Ui[v] + Uj[v]);
+    // these scalars only shape the projection: ordinary (contracted) arithmetic
+    double rho, Y[NS], uu[3], e, vol;
+    decode<NS, D, false>(Ui, rho, Y, uu, e, vol);
+    double p, T, a, al, be;
+    // the Newton start of several stiffened liquids: the mean of the two
+    // cells' pressures, close to the averaged state's
+    pt_equilibrium<NS, false>(P, Y, e, vol, p, T, rho,
+                              0.5 * (wget(P, Wc, P.wP, ri) + wget(P, Wc, P.wP, rj)));
+    eos_char<NS>(P, Y, p, T, rho, a, al, be);
+    X = (rho * a * a * be - 1.0) / (al * a * a * rho);
+    c = a * rho;
+    ic = 1.0 / c;
+  }
+
+  // steps 2-3: project, interpolate both sides (WENO5-Z unless RC says
+  // otherwise), back to physical space
+  double YL[NS], YR[NS], uL[3] = {0.0, 0.0, 0.0}, uR[3] = {0.0, 0.0, 0.0}, PL, PR, TL, TR;
+  {
+    double w1[6], w5[6], w6[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      const double T = wget(P, Wc, P.wT, cr[j]);
+      const double p = wget(P, Wc, P.wP, cr[j]);
+      const double un = wget(P, Wc, P.wU + d, cr[j]) * sgn_flip(cr[j].flip, d);
+      w1[j] = T - X * p;
+      w5[j] = (0.5 * c) * un + 0.5 * p;
+      w6[j] = (-0.5 * c) * un + 0.5 * p;
+    }
+    double w1L, w1R, w5L, w5R, w6L, w6R;
+    fast::recon_lr<RC>(P, w1, w1L, w1R);
+    fast::recon_lr<RC>(P, w5, w5L, w5R);
+    fast::recon_lr<RC>(P, w6, w6L, w6R);
+    TL = w1L + X * w5L + X * w6L;
+    TR = w1R + X * w5R + X * w6R;
+    uL[d] = ic * w5L + (-ic) * w6L;
+    uR[d] = ic * w5R + (-ic) * w6R;
+    PL = w5L + w6L;
+    PR = w5R + w6R;
+  }
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    double y[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) y[j] = wget(P, Wc, P.wY + k, cr[j]);
+    fast::recon_lr<RC>(P, y, YL[k], YR[k]);
+  }
+#pragma unroll
+  for (int t = 0; t < D; ++t) {
+    if (t == d) continue;
+    double y[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) y[j] = wget(P, Wc, P.wU + t, cr[j]) * sgn_flip(cr[j].flip, t);
+    fast::recon_lr<RC>(P, y, uL[t], uR[t]);
+  }
+
+  // cell values of the two face neighbours
+  double Yi[NS], Yj[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    Yi[k] = wget(P, Wc, P.wY + k, ri);
+    Yj[k] = wget(P, Wc, P.wY + k, rj);
+  }
+  const double Ti = wget(P, Wc, P.wT, ri), Tj = wget(P, Wc, P.wT, rj);
+  const double Pi = wget(P, Wc, P.wP, ri), Pj = wget(P, Wc, P.wP, rj);
+
+  // interpolation limiters (Sec. 3.3.1)
+  if (P.pos_limiter) {
+    if (y_limiter<NS>(YL, Yi)) fl |= F_YLIM_L;
+    if (y_limiter<NS>(YR, Yj)) fl |= F_YLIM_R;
+    if (!positive(TL)) { TL = Ti; fl |= F_THETA_T_L; }
+    if (!positive(TR)) { TR = Tj; fl |= F_THETA_T_R; }
+    bool okL = true, okR = true;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      if (positive(YL[k]) && !positive(PL + P.pinf[k])) okL = false;
+      if (positive(YR[k]) && !positive(PR + P.pinf[k])) okR = false;
+    }
+    if (!okL) { PL = Pi; fl |= F_THETA_P_L; }
+    if (!okR) { PR = Pj; fl |= F_THETA_P_R; }
+  }
+
+  // steps 4-6: face EOS, conserved face states, HLLC
+  double Fx[NV];
+  {
+    State<NS> sL, sR;
+    state_from_primitive<NS>(P, YL, uL, PL, TL, sL);
+    state_from_primitive<NS>(P, YR, uR, PR, TR, sR);
+    hllc<NS, D>(d, sL, sR, Fx);
+  }
+
+  // flux limiter (Sec. 3.3.2): pseudo-updates of both cells
+  // Bi, Bj: the RK combination rk0 U^n + rk1 U^(k) of both cells, formed
+  // once for the (up to three) pseudo-update tests of this face
+  double Bi[NV], Bj[NV], Uki[NV], Ukj[NV];
+  const double lam = 2.0 * D * rk2 * dt * P.inv_dx;
+  if (P.pos_limiter || P.cdi) {
+    load_U<NS, D>(P, Uk, Uin, ri, Uki);
+    load_U<NS, D>(P, Uk, Uin, rj, Ukj);
+    load_U<NS, D>(P, Un, P.gn, ri, Bi);
+    load_U<NS, D>(P, Un, P.gn, rj, Bj);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      Bi[v] = rk0 * Bi[v] + rk1 * Uki[v];
+      Bj[v] = rk0 * Bj[v] + rk1 * Ukj[v];
+    }
+  }
+  auto passes = [&](const double* Ft) {
+    double Ti_[NV], Tj_[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      Ti_[v] = Bi[v] - lam * Ft[v];
+      Tj_[v] = Bj[v] + lam * Ft[v];
+    }
+    return admissible<NS, D>(P, Ti_) && admissible<NS, D>(P, Tj_);
+  };
+  if (P.pos_limiter && !passes(Fx)) {
+    State<NS> si, sj;
+    si.rho = wget(P, Wc, P.wRho, ri);
+    sj.rho = wget(P, Wc, P.wRho, rj);
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      si.rhoY[k] = Uki[k];
+      sj.rhoY[k] = Ukj[k];
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      si.u[t] = t < D ? wget(P, Wc, P.wU + t, ri) * sgn_flip(ri.flip, t) : 0.0;
+      sj.u[t] = t < D ? wget(P, Wc, P.wU + t, rj) * sgn_flip(rj.flip, t) : 0.0;
+      si.m[t] = t < D ? Uki[NS + t] : 0.0;
+      sj.m[t] = t < D ? Ukj[NS + t] : 0.0;
+    }
+    si.p = Pi;
+    sj.p = Pj;
+    si.E = Uki[NS + D];
+    sj.E = Ukj[NS + D];
+    si.a = wget(P, Wc, P.wA, ri);
+    sj.a = wget(P, Wc, P.wA, rj);
+    hllc<NS, D>(d, si, sj, Fx);
+    fl |= F_HLLC_FALLBACK;
+  }
+
+  // interface regularization (Sec. 3.2), KEEP split form, with its limiter
+  if (P.cdi && P.two_phase) {
+    bool pres_i[2] = {false, false}, pres_j[2] = {false, false};
+    {
+      // (branches on the phase rather than ypi[P.phase[k]]: an array indexed
+      // at run time would live on the stack)
+      double ypi[2] = {0.0, 0.0}, ypj[2] = {0.0, 0.0};
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        if (P.phase[k]) {
+          ypi[1] += Yi[k];
+          ypj[1] += Yj[k];
+        } else {
+          ypi[0] += Yi[k];
+          ypj[0] += Yj[k];
+        }
+      }
+#pragma unroll
+      for (int ph = 0; ph < 2; ++ph) {
+        pres_i[ph] = ypi[ph] >= ABSENT;
+        pres_j[ph] = ypj[ph] >= ABSENT;
+      }
+    }
+    if ((pres_i[0] || pres_j[0]) && (pres_i[1] || pres_j[1])) {
+      const double ceps = P.cdi_eps;
+      const double psi_i = wget(P, Wc, P.wPsi, ri), psi_j = wget(P, Wc, P.wPsi, rj);
+      const double dphi = (wget(P, Wc, P.wPhi0, rj) - wget(P, Wc, P.wPhi0, ri)) * P.inv_dx;
+      double g[3] = {0.0, 0.0, 0.0};
+      g[d] = (psi_j - psi_i) * P.inv_dx;
+#pragma unroll
+      for (int t = 0; t < D; ++t) {
+        if (t == d) continue;
+        int a0[3] = {ci[0], ci[1], ci[2]}, a1[3] = {ci[0], ci[1], ci[2]};
+        int b0[3] = {ci[0], ci[1], ci[2]}, b1[3] = {ci[0], ci[1], ci[2]};
+        a0[t] += 1;
+        a1[t] -= 1;
+        b0[t] += 1;
+        b1[t] -= 1;
+        b0[d] += 1;
+        b1[d] += 1;
+        const double pip = wget(P, Wc, P.wPsi, map_cell_dt<d>(P, t, a0[0], a0[1], a0[2]));
+        const double pim = wget(P, Wc, P.wPsi, map_cell_dt<d>(P, t, a1[0], a1[1], a1[2]));
+        const double pjp = wget(P, Wc, P.wPsi, map_cell_dt<d>(P, t, b0[0], b0[1], b0[2]));
+        const double pjm = wget(P, Wc, P.wPsi, map_cell_dt<d>(P, t, b1[0], b1[1], b1[2]));
+        g[t] = 0.5 * ((pip - pim) * (0.5 * P.inv_dx) + (pjp - pjm) * (0.5 * P.inv_dx));
+      }
+      const double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+      const double nd = gn >= GTOL ? g[d] / gn : 0.0;
+      // 1 - tanh^2 as 1 / cosh^2 (no cancellation near the phi_min floor)
+      const double ch = cosh((0.5 * (psi_i + psi_j)) / (2.0 * ceps));
+      const double sech2 = 1.0 / (ch * ch);
+      const double ahat0 = Gamma * (ceps * dphi - 0.25 * (sech2 - P.sharp0) * nd);
+      double Fdi[NV], Rtot = 0.0, hR = 0.0;
+#pragma unroll
+      for (int ph = 0; ph < 2; ++ph) {
+        const double ahat = ph == 0 ? ahat0 : -ahat0;
+        const bool pi = pres_i[ph], pj = pres_j[ph];
+        auto keep = [&](double a, double b) { return pi && pj ? 0.5 * (a + b) : (pi ? a : (pj ? b : 0.0)); };
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+          if (P.phase[k] != ph) continue;
+          const double R = -keep(wget(P, Wc, P.wYrho + k, ri), wget(P, Wc, P.wYrho + k, rj)) * ahat;
+          Fdi[k] = R;
+          Rtot += R;
+        }
+        hR -= keep(wget(P, Wc, P.wHrho + ph, ri), wget(P, Wc, P.wHrho + ph, rj)) * ahat;
+      }
+      double kb = 0.0;
+#pragma unroll
+      for (int t = 0; t < D; ++t) {
+        const double ui = wget(P, Wc, P.wU + t, ri) * sgn_flip(ri.flip, t);
+        const double uj = wget(P, Wc, P.wU + t, rj) * sgn_flip(rj.flip, t);
+        kb += ui * uj;
+        Fdi[NS + t] = 0.5 * (ui + uj) * Rtot;
+      }
+      Fdi[NS + D] = 0.5 * kb * Rtot + hR;
+      double Ft[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Ft[v] = Fx[v] + Fdi[v];
+      if (P.pos_limiter && !passes(Ft)) {
+        fl |= F_CDI_DROPPED;
+      } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Fx[v] = Ft[v];
+      }
+    }
+  }
+
+  // diffusive flux F_nu: species diffusion (Eq. SpeciesMassDiffusion),
+  // viscous stress and heat conduction.  It passes the same flux limiter as
+  // the regularization flux: added to the admissible flux when both
+  // pseudo-updates stay admissible, else not added at this face.
+  double Fnu[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) Fnu[v] = 0.0;
+  if (P.diffusion) {
+    const double rb = 0.5 * (wget(P, Wc, P.wRho, ri) + wget(P, Wc, P.wRho, rj));
+    double Jh = 0.0;
+#pragma unroll
+    for (int ph = 0; ph < 2; ++ph) {
+      double Yp = 0.0, S = 0.0, Bf[NS], G[NS];
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        Bf[k] = 0.0;
+        G[k] = 0.0;
+        if (P.phase[k] != ph) continue;
+        Yp += 0.5 * (Yi[k] + Yj[k]);
+        Bf[k] = 0.5 * (wget(P, Wc, P.wB + k, ri) + wget(P, Wc, P.wB + k, rj));
+        G[k] = (wget(P, Wc, P.wXr + k, rj) - wget(P, Wc, P.wXr + k, ri)) * P.inv_dx;
+        S += Bf[k] * G[k];
+      }
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        if (P.phase[k] != ph) continue;
+        const double J = -rb * (Yp * Bf[k] * G[k] - 0.5 * (Yi[k] + Yj[k]) * S);
+        Fnu[k] = J;
+        Jh += J * (0.5 * (h_k(P, k, Pi, Ti) + h_k(P, k, Pj, Tj)));
+      }
+    }
+    Fnu[NS + D] = Jh;
+  }
+
+  // viscous stress and heat conduction (Eq. DiffusionTerms), second-order
+  // central: face averages of the two cells, normal derivative
+  // (q_j - q_i)/dx, a tangential one the mean of the two cells' central
+  // differences; the energy row carries -u.tau + q
+  if (P.viscous) {
+    double gu[3][3];  // gu[i][j] = d u_i / d x_j on the face
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) gu[i][j] = 0.0;
+    double ui[3] = {0.0, 0.0, 0.0}, uj[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      ui[i] = wget(P, Wc, P.wU + i, ri) * sgn_flip(ri.flip, i);
+      uj[i] = wget(P, Wc, P.wU + i, rj) * sgn_flip(rj.flip, i);
+      gu[i][d] = (uj[i] - ui[i]) * P.inv_dx;
+    }
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+      if (t == d) continue;
+      int a0[3] = {ci[0], ci[1], ci[2]}, a1[3] = {ci[0], ci[1], ci[2]};
+      a0[t] += 1;
+      a1[t] -= 1;
+      int b0[3] = {a0[0], a0[1], a0[2]}, b1[3] = {a1[0], a1[1], a1[2]};
+      b0[d] += 1;
+      b1[d] += 1;
+      const CRef ip = map_cell_dt<d>(P, t, a0[0], a0[1], a0[2]), im = map_cell_dt<d>(P, t, a1[0], a1[1], a1[2]);
+      const CRef jp = map_cell_dt<d>(P, t, b0[0], b0[1], b0[2]), jm = map_cell_dt<d>(P, t, b1[0], b1[1], b1[2]);
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        const double dip = wget(P, Wc, P.wU + i, ip) * sgn_flip(ip.flip, i) -
+                           wget(P, Wc, P.wU + i, im) * sgn_flip(im.flip, i);
+        const double djp = wget(P, Wc, P.wU + i, jp) * sgn_flip(jp.flip, i) -
+                           wget(P, Wc, P.wU + i, jm) * sgn_flip(jm.flip, i);
+        gu[i][t] = 0.25 * P.inv_dx * (dip + djp);
+      }
+    }
+    double div = 0.0;
+#pragma unroll
+    for (int k = 0; k < D; ++k) div += gu[k][k];
+    const double mub = 0.5 * (wget(P, Wc, P.wMu, ri) + wget(P, Wc, P.wMu, rj));
+    const double lamb = 0.5 * (wget(P, Wc, P.wLam, ri) + wget(P, Wc, P.wLam, rj));
+    double work = 0.0;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      const double tau = mub * (gu[i][d] + gu[d][i] - (i == d ? (2.0 / 3.0) * div : 0.0));
+      Fnu[NS + i] = -tau;
+      work += 0.5 * (ui[i] + uj[i]) * tau;
+    }
+    Fnu[NS + D] -= work + lamb * (Tj - Ti) * P.inv_dx;
+  }
+  if (P.diffusion || P.viscous) {
+    double Ft[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Ft[v] = Fx[v] + Fnu[v];
+    if (P.pos_limiter && !passes(Ft)) {
+      fl |= F_DIFF_DROPPED;
+    } else {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Fx[v] = Ft[v];
+    }
+  }
+
+#pragma unroll
+  for (int v = 0; v < NV; ++v) F[(long long)v * nf + fid] = Fx[v];
+  if (flags) flags[fid] = fl;
+  if (stats && fl) {
+    if (fl & F_HLLC_FALLBACK) atomicAdd(stats + 1, 1ull);
+    if (fl & F_CDI_DROPPED) atomicAdd(stats + 2, 1ull);
+    if (fl & (F_THETA_P_L | F_THETA_P_R)) atomicAdd(stats + 3, 1ull);
+    if (fl & (F_THETA_T_L | F_THETA_T_R)) atomicAdd(stats + 4, 1ull);
+    if (fl & (F_YLIM_L | F_YLIM_R)) atomicAdd(stats + 5, 1ull);
+    if (fl & F_DIFF_DROPPED) atomicAdd(stats + 6, 1ull);
+  }
+}
+
+// the forward FP64 face pass of one direction with interpolation RC
+template <int NS, int D, int RC>
+struct FaceImpl {
+  static void face(const KParams& P, cudaStream_t s, int d, const double* Wc, const double* Un, const double* Uk,
+                   const double* Uin, const double* scal, double rk0, double rk1, double rk2, double* F,
+                   uint32_t* flags, unsigned long long* stats) {
+    long long nf = 1;
+    for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
+    const unsigned nb = nblocks(nf, FACE_THREADS);
+    if (d == 0)
+      fast::k_face<NS, D, 0, RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F, flags, stats);
+    else if (d == 1)
+      fast::k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+                                                                     flags, stats);
+    else
+      fast::k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+                                                                     flags, stats);
+  }
+};
+
+// the face pass of interpolation RC for (dimension, species count), or null
+template <int RC>
+FaceFn face(int dim, int ns) {
+  switch (dim * 8 + ns) {
+    case 9: return &FaceImpl<1, 1, RC>::face;
+    case 10: return &FaceImpl<2, 1, RC>::face;
+    case 11: return &FaceImpl<3, 1, RC>::face;
+    case 12: return &FaceImpl<4, 1, RC>::face;
+    case 17: return &FaceImpl<1, 2, RC>::face;
+    case 18: return &FaceImpl<2, 2, RC>::face;
+    case 19: return &FaceImpl<3, 2, RC>::face;
+    case 20: return &FaceImpl<4, 2, RC>::face;
+    case 25: return &FaceImpl<1, 3, RC>::face;
+    case 26: return &FaceImpl<2, 3, RC>::face;
+    case 27: return &FaceImpl<3, 3, RC>::face;
+    case 28: return &FaceImpl<4, 3, RC>::face;
+    default: return nullptr;
+  }
+}
+
+}  // namespace fast
+}  // namespace mpmc

@@ -96,7 +96,8 @@ extern "C" int mpmc_rhs_noalloc(const mpmc_grid* grid, const mpmc_eos* eos, cons
   // an error left pending by earlier work of the caller is reported as it
   // is and not cleared: the final check below then only sees this call's
   if (cudaPeekAtLastError() != cudaSuccess) return MPMC_CUDA_ERROR;
-  const Ops ops = P.dim == 1 ? ops_fp64_d1(P.ns) : (P.dim == 2 ? ops_fp64_d2(P.ns) : ops_fp64_d3(P.ns));
+  Ops ops = P.dim == 1 ? ops_fp64_d1(P.ns) : (P.dim == 2 ? ops_fp64_d2(P.ns) : ops_fp64_d3(P.ns));
+  ops.face = face_fast_weno5z(P.dim, P.ns);
   if (!ops.face) return MPMC_INVALID_ARG;
   void* base = nullptr;
   rc = scratch_address(&base);

@@ -48,6 +48,15 @@ using FaceFn = decltype(Ops::face);
 FaceFn face_fp64_weno5js(int dim, int ns);
 FaceFn face_fp64_teno5(int dim, int ns);
 FaceFn face_fp64_teno6(int dim, int ns);
+// forward FP64 face passes (float-float interpolation weights), the ones that
+// steps and right-hand sides run: mpmc_fast_d{1,2,3}.cu,
+// mpmc_fast_{weno5js,teno5,teno6}.cu
+FaceFn face_fast_d1(int ns);
+FaceFn face_fast_d2(int ns);
+FaceFn face_fast_d3(int ns);
+FaceFn face_fast_weno5js(int dim, int ns);
+FaceFn face_fast_teno5(int dim, int ns);
+FaceFn face_fast_teno6(int dim, int ns);
 // the same for mixed-precision contexts: mpmc_mixed_recon_{weno5js,teno5,teno6}.cu
 FaceFn face_mixed_weno5js(int dim, int ns);
 FaceFn face_mixed_teno5(int dim, int ns);
@@ -59,6 +68,10 @@ using AdjFaceFn = decltype(AdjOps::face);
 AdjFaceFn adj_face_weno5js(int dim, int ns);
 AdjFaceFn adj_face_teno5(int dim, int ns);
 AdjFaceFn adj_face_teno6(int dim, int ns);
+
+inline FaceFn face_fast_weno5z(int dim, int ns) {
+  return dim == 1 ? face_fast_d1(ns) : (dim == 2 ? face_fast_d2(ns) : face_fast_d3(ns));
+}
 
 // per-dimension tables, defined in mpmc_kernels_d{1,2,3}.cu (FP64) and
 // mpmc_mixed_d{1,2,3}.cu (mixed precision; init is the FP64 one)

@@ -90,6 +90,14 @@ inline int build_params(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_mode
     }
   P.two_phase = has0 && has1;
   P.weno_eps = m->weno_eps;
+  {
+    // (without an epsilon: one below every scale, the float-float form's floor)
+    int e = -4000;
+    const double f = m->weno_eps > 0.0 ? 2.0 * std::frexp(4.0 * m->weno_eps, &e) : 1.0;
+    P.weno_eps4.h = (float)f;
+    P.weno_eps4.l = (float)(f - (double)P.weno_eps4.h);
+    P.weno_eps4.e = e - 1;
+  }
   P.cdi = m->cdi ? 1 : 0;
   P.diffusion = m->diffusion ? 1 : 0;
   P.pos_limiter = m->pos_limiter ? 1 : 0;
