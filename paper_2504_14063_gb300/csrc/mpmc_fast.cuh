@@ -32,28 +32,160 @@ static __device__ __noinline__ double2 weno5z_lr_fp64(double w0, double w1, doub
   return make_double2(L, R);
 }
 
+// Out of line: a face interpolates nine fields (3D, four species), and the code
+// of all of them inlined (17,000 instructions of a face) does not fit the
+// instruction caches; the pass then waited for instructions three times as
+// long as it issued them (droplet field 128^3, faces of a step: 46.4 ms
+// inlined, 39.3 ms with this function called, 33.8 ms with the face states
+// and the limiter's tests called too).
+static __device__ __noinline__ double2 weno5z_lr(double w0, double w1, double w2, double w3, double w4, double w5, float eh, float el,
+                              int ee) {
+  const double w[6] = {w0, w1, w2, w3, w4, w5};
+  double L, R;
+  if (weno5z_lr_ff(w, WenoEps{eh, el, ee}, L, R)) return make_double2(L, R);
+  return weno5z_lr_fp64(w0, w1, w2, w3, w4, w5, 0.25 * scalbn((double)eh + (double)el, ee));
+}
+
 // both face values of one field from the cells y[0..5] = i-2..i+3 around
-// the face i+1/2; WENO5-Z in float-float (mpmc_ff.h)
-template <int RC>
+// the face i+1/2; WENO5-Z in float-float (mpmc_ff.h).  TWICE: the field is
+// twice the method's (eps, compared with its square, then counts four times).
+template <int RC, bool TWICE = false>
 __device__ __forceinline__ void recon_lr(const KParams& P, const double* y, double& L, double& R) {
   if constexpr (RC == RC_WENO5Z) {
-    if (!weno5z_lr_ff(y, P.weno_eps4, L, R)) {
-      const double2 v = weno5z_lr_fp64(y[0], y[1], y[2], y[3], y[4], y[5], P.weno_eps);
-      L = v.x;
-      R = v.y;
-    }
+    const double2 v = weno5z_lr(y[0], y[1], y[2], y[3], y[4], y[5], P.weno_eps4.h, P.weno_eps4.l,
+                                P.weno_eps4.e + (TWICE ? 2 : 0));
+    L = v.x;
+    R = v.y;
+  } else if constexpr (TWICE) {
+    double h[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) h[j] = 0.5 * y[j];
+    mpmc::recon_lr<RC>(h, P.weno_eps, L, R);
+    L *= 2.0;
+    R *= 2.0;
   } else {
     mpmc::recon_lr<RC>(y, P.weno_eps, L, R);
   }
 }
 
 // ---------------------------------------------------------------------------
+// The flux limiter's tests on the FP32 pipe (the FP64 path).  A pseudo-update
+// T = B + s F (B = rk0 U^n + rk1 U^(k)) is first tested on FP32 roundings: a
+// test is decided there only when its value clears LIM_MARGIN times the
+// magnitudes of its terms, 100 times what FP32 rounding can move it, and
+// when it is far from FP32 underflow; so a decision is the FP64 test's own.
+// 1: admissible, 0: not, -1: too close to call (also overflow and NaN).
+constexpr float LIM_MARGIN = 1e-4f;
+constexpr float LIM_TINY = 1e-20f;
+
+// B (value) and M (sum of its terms' magnitudes) of one cell in FP32
+template <int NS, int D>
+__device__ __forceinline__ void limiter_base(const KParams& P, const double* __restrict__ Un,
+                                             const double* __restrict__ Uk, const double* __restrict__ Gk,
+                                             const CRef r, const float rk0, const float rk1, float* B, float* M) {
+  constexpr int NV = NS + D + 1;
+  const bool ghost = r.idx >= P.ncell;
+  const double* un = ghost ? P.gn + (r.idx - P.ncell) : Un + r.idx;
+  const double* uk = ghost ? Gk + (r.idx - P.ncell) : Uk + r.idx;
+  const long long st = ghost ? P.gstride : P.ncell;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    float a = rk0 * narrow(un[(long long)v * st]);
+    float b = rk1 != 0.f ? rk1 * narrow(uk[(long long)v * st]) : 0.f;
+    if (v >= NS && v < NS + D && ((r.flip >> (v - NS)) & 1u)) {
+      a = -a;
+      b = -b;
+    }
+    B[v] = a + b;
+    M[v] = fabsf(a) + fabsf(b);
+  }
+}
+
+template <int NS, int D>
+__device__ __noinline__ int admissible_fp32(const KParams& P, const float* B, const float* M, const float* F,
+                                               const float s) {
+  constexpr int NV = NS + D + 1;
+  float T[NV], G[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const float f = s * F[v];
+    T[v] = B[v] + f;
+    G[v] = M[v] + fabsf(f);
+  }
+  bool undecided = false;
+  auto test = [&](float val, float mag) {
+    if (val > LIM_MARGIN * mag) return true;
+    if (!(val < -LIM_MARGIN * mag)) undecided = true;
+    return false;
+  };
+  float rho = 0.f, Grho = 0.f;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    rho += T[k];
+    Grho += G[k];
+  }
+  bool ok = test(rho, Grho);
+  float sq = 0.f, Gsq = 0.f;
+  if (P.has_b) {
+    float sb = 0.f, Gsb = 1.f;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      sb += T[k] * P.f32.b[k];
+      Gsb += G[k] * fabsf(P.f32.b[k]);
+    }
+    ok = test(1.f - sb, Gsb) && ok;
+  }
+  if (P.has_q) {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      sq += T[k] * P.f32.q[k];
+      Gsq += G[k] * fabsf(P.f32.q[k]);
+    }
+  }
+  const float yt = (float)YTOL;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) ok = test(T[k] + yt * rho, G[k] + yt * Grho) && ok;
+  float mm = 0.f, Gmm = 0.f;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    mm += T[NS + d] * T[NS + d];
+    Gmm += G[NS + d] * G[NS + d];
+  }
+  const float Ge = Grho * G[NS + D] + 0.5f * Gmm + Grho * Gsq;
+  ok = test(rho * T[NS + D] - 0.5f * mm - rho * sq, Ge) && ok;
+  // terms near FP32's underflow are not judged by their FP32 magnitudes
+  if (!(Grho > LIM_TINY && Ge > LIM_TINY && fabsf(s) > LIM_TINY)) return -1;
+  if (ok) return 1;
+  // a test decided "no" makes the state inadmissible whatever the others say
+  return undecided ? -1 : 0;
+}
+
+// the FP64 test of T = rk0 U^n + rk1 U^(k) + s F, for a flux that the FP32
+// one could not decide: out of line and from memory, so that it costs the
+// face kernel no registers
+template <int NS, int D>
+__device__ __noinline__ bool admissible_fp64(const KParams& P, const double* Un, const double* Uk, const double* Gk,
+                                             const CRef r, const double* F, const double rk0, const double rk1,
+                                             const double s) {
+  constexpr int NV = NS + D + 1;
+  double T[NV], B[NV];
+  load_U<NS, D>(P, Un, P.gn, r, B);
+  load_U<NS, D>(P, Uk, Gk, r, T);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) T[v] = rk0 * B[v] + rk1 * T[v] + s * F[v];
+  return admissible<NS, D>(P, T);
+}
+
+// ---------------------------------------------------------------------------
 // DIR: the face direction, a template parameter so that every array indexed
 // by it is indexed by a constant (registers, not the stack).  RC: the
 // ENO-type interpolation (RC_WENO5Z, the method's, or one of Sec. 4.1's others)
+// Four blocks per SM (128 registers): more warps hide the latencies of the
+// FP64 and FP32 chains (three or two blocks, unbounded registers: 20 % slower;
+// five and six, with spills: within 5 % either way).
 template <int NS, int D, int DIR, int RC>
-__global__ void __launch_bounds__(FACE_THREADS)
-    k_face(const KParams P, const double* __restrict__ Wc, const double* __restrict__ Un,
+__global__ void __launch_bounds__(FACE_THREADS, 4)
+    k_face(const __grid_constant__ KParams P, const double* __restrict__ Wc, const double* __restrict__ Un,
            const double* __restrict__ Uk, const double* __restrict__ Uin, const double* __restrict__ scal,
            const double rk0, const double rk1, const double rk2, double* __restrict__ F,
            uint32_t* __restrict__ flags, unsigned long long* __restrict__ stats) {
@@ -68,7 +200,8 @@ __global__ void __launch_bounds__(FACE_THREADS)
   int ci[3] = {fc[0], fc[1], fc[2]};
   ci[d] -= 1;  // the cell on the low side of the face
   const double dt = scal[0], Gamma = scal[1];
-  const long long ws = P.wstride;
+  // FP32 roundings for the limiter's tests
+  const float rk0f = narrow(rk0), rk1f = narrow(rk1), rk2f = narrow(rk2), dtdx = narrow(dt) * P.f32.inv_dx;
 
   CRef cr[6];
 #pragma unroll
@@ -179,32 +312,35 @@ __global__ void __launch_bounds__(FACE_THREADS)
     hllc<NS, D>(d, sL, sR, Fx);
   }
 
-  // flux limiter (Sec. 3.3.2): pseudo-updates of both cells
-  // Bi, Bj: the RK combination rk0 U^n + rk1 U^(k) of both cells, formed
-  // once for the (up to three) pseudo-update tests of this face
-  double Bi[NV], Bj[NV], Uki[NV], Ukj[NV];
-  const double lam = 2.0 * D * rk2 * dt * P.inv_dx;
-  if (P.pos_limiter || P.cdi) {
-    load_U<NS, D>(P, Uk, Uin, ri, Uki);
-    load_U<NS, D>(P, Uk, Uin, rj, Ukj);
-    load_U<NS, D>(P, Un, P.gn, ri, Bi);
-    load_U<NS, D>(P, Un, P.gn, rj, Bj);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      Bi[v] = rk0 * Bi[v] + rk1 * Uki[v];
-      Bj[v] = rk0 * Bj[v] + rk1 * Ukj[v];
-    }
+  // flux limiter (Sec. 3.3.2): pseudo-updates of both cells, tested on the
+  // FP32 pipe with a margin and in FP64 where that cannot decide.  The up to
+  // three tests of a face were a tenth of its FP64 operations.
+  float Bi[NV], Bj[NV], Mi[NV], Mj[NV];
+  const float lamf = (float)(2 * D) * (rk2f * dtdx);
+  if (P.pos_limiter) {
+    limiter_base<NS, D>(P, Un, Uk, Uin, ri, rk0f, rk1f, Bi, Mi);
+    limiter_base<NS, D>(P, Un, Uk, Uin, rj, rk0f, rk1f, Bj, Mj);
   }
   auto passes = [&](const double* Ft) {
-    double Ti_[NV], Tj_[NV];
+    float Ff[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      Ti_[v] = Bi[v] - lam * Ft[v];
-      Tj_[v] = Bj[v] + lam * Ft[v];
-    }
-    return admissible<NS, D>(P, Ti_) && admissible<NS, D>(P, Tj_);
+    for (int v = 0; v < NV; ++v) Ff[v] = narrow(Ft[v]);
+    const int a = admissible_fp32<NS, D>(P, Bi, Mi, Ff, -lamf);
+    if (a == 0) return false;
+    const int b = admissible_fp32<NS, D>(P, Bj, Mj, Ff, lamf);
+    if (b == 0) return false;
+    if (a == 1 && b == 1) return true;
+    const double lam = 2.0 * D * rk2 * dt * P.inv_dx;
+    double tmp[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) tmp[v] = Ft[v];
+    return admissible_fp64<NS, D>(P, Un, Uk, Uin, ri, tmp, rk0, rk1, -lam) &&
+           admissible_fp64<NS, D>(P, Un, Uk, Uin, rj, tmp, rk0, rk1, lam);
   };
   if (P.pos_limiter && !passes(Fx)) {
+    double Uki[NV], Ukj[NV];
+    load_U<NS, D>(P, Uk, Uin, ri, Uki);
+    load_U<NS, D>(P, Uk, Uin, rj, Ukj);
     State<NS> si, sj;
     si.rho = wget(P, Wc, P.wRho, ri);
     sj.rho = wget(P, Wc, P.wRho, rj);
