@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "mpmc_avg.h"
 #include "mpmc_ff.h"
 #include "mpmc_narrow.h"
 
@@ -74,6 +75,7 @@ struct KParams {
   } f32;
   // read by the forward FP64 passes (mpmc_fast.cuh)
   WenoEps weno_eps4;  // 4 weno_eps, for the float-float WENO5-Z
+  SpeciesFF sff[MAXS];       // Rk, cv, cp, pinf as float-floats
 };
 
 // fills P.f32 from the FP64 fields (host)

@@ -177,6 +177,42 @@ __device__ __noinline__ bool admissible_fp64(const KParams& P, const double* Un,
 }
 
 // ---------------------------------------------------------------------------
+// partial densities of a mapped cell (as load_U)
+template <int NS>
+__device__ __forceinline__ void load_rhoY(const KParams& P, const double* __restrict__ U,
+                                          const double* __restrict__ G, CRef r, double* out) {
+  const bool ghost = r.idx >= P.ncell;
+  const double* p = ghost ? G + (r.idx - P.ncell) : U + r.idx;
+  const long long st = ghost ? P.gstride : P.ncell;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) out[k] = p[(long long)k * st];
+}
+
+// X and c of the averaged state in FP64: the p-T equilibrium of the averaged
+// conserved vector, for faces whose float-float solve (face_avg_ff) does not
+// settle or leaves its range; out of line, so that it costs the face kernel
+// no registers
+template <int NS, int D>
+__device__ __noinline__ double2 face_avg_fp64(const KParams& P, const double* Wc, const double* Uk, const double* Uin,
+                                              const CRef ri, const CRef rj) {
+  constexpr int NV = NS + D + 1;
+  double Ui[NV], Uj[NV];
+  load_U<NS, D>(P, Uk, Uin, ri, Ui);
+  load_U<NS, D>(P, Uk, Uin, rj, Uj);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) Ui[v] = 0.5 * (Ui[v] + Uj[v]);
+  // these scalars only shape the projection: ordinary (contracted) arithmetic
+  double rho, Y[NS], uu[3], e, vol, p, T, a, al, be;
+  decode<NS, D, false>(Ui, rho, Y, uu, e, vol);
+  // the Newton start of several stiffened liquids: the mean of the two
+  // cells' pressures, close to the averaged state's
+  pt_equilibrium<NS, false>(P, Y, e, vol, p, T, rho,
+                            0.5 * (wget(P, Wc, P.wP, ri) + wget(P, Wc, P.wP, rj)));
+  eos_char<NS>(P, Y, p, T, rho, a, al, be);
+  return make_double2((rho * a * a * be - 1.0) / (al * a * a * rho), a * rho);
+}
+
+// ---------------------------------------------------------------------------
 // DIR: the face direction, a template parameter so that every array indexed
 // by it is indexed by a constant (registers, not the stack).  RC: the
 // ENO-type interpolation (RC_WENO5Z, the method's, or one of Sec. 4.1's others)
@@ -213,27 +249,25 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   const CRef ri = cr[2], rj = cr[3];
   uint32_t fl = 0u;
 
-  // step 1: averaged conserved state on the face, its EOS, the scalars of
-  // the characteristic matrices (Appendix A)
+  // step 1: the scalars of the characteristic matrices (Appendix A) at the
+  // averaged conserved state
   double X, c, ic;
   {
-    double Ui[NV], Uj[NV];
-    load_U<NS, D>(P, Uk, Uin, ri, Ui);
-    load_U<NS, D>(P, Uk, Uin, rj, Uj);
+    double mi[NS], mj[NS], ui[3] = {0.0, 0.0, 0.0}, uj[3] = {0.0, 0.0, 0.0};
+    load_rhoY<NS>(P, Uk, Uin, ri, mi);
+    load_rhoY<NS>(P, Uk, Uin, rj, mj);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) Ui[v] = 0.5 * (Ui[v] + Uj[v]);
-    // these scalars only shape the projection: ordinary (contracted) arithmetic
-    double rho, Y[NS], uu[3], e, vol;
-    decode<NS, D, false>(Ui, rho, Y, uu, e, vol);
-    double p, T, a, al, be;
-    // the Newton start of several stiffened liquids: the mean of the two
-    // cells' pressures, close to the averaged state's
-    pt_equilibrium<NS, false>(P, Y, e, vol, p, T, rho,
-                              0.5 * (wget(P, Wc, P.wP, ri) + wget(P, Wc, P.wP, rj)));
-    eos_char<NS>(P, Y, p, T, rho, a, al, be);
-    X = (rho * a * a * be - 1.0) / (al * a * a * rho);
-    c = a * rho;
-    ic = 1.0 / c;
+    for (int t = 0; t < D; ++t) {
+      ui[t] = wget(P, Wc, P.wU + t, ri) * sgn_flip(ri.flip, t);
+      uj[t] = wget(P, Wc, P.wU + t, rj) * sgn_flip(rj.flip, t);
+    }
+    if (!face_avg_ff<NS, D>(P.sff, mi, mj, wget(P, Wc, P.wP, ri), wget(P, Wc, P.wP, rj), wget(P, Wc, P.wT, ri),
+                            wget(P, Wc, P.wT, rj), ui, uj, X, c, ic)) {
+      const double2 v = face_avg_fp64<NS, D>(P, Wc, Uk, Uin, ri, rj);
+      X = v.x;
+      c = v.y;
+      ic = 1.0 / c;
+    }
   }
 
   // steps 2-3: project, interpolate both sides (WENO5-Z unless RC says

@@ -77,6 +77,16 @@ inline int build_params(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_mode
     P.Sc[k] = eos->Sc[k];
     P.Rk[k] = (eos->gamma[k] - 1.0) * eos->cv[k];
     P.cp[k] = eos->gamma[k] * eos->cv[k];
+    auto split = [](double x) {
+      ff r;
+      r.h = (float)x;
+      r.l = (float)(x - (double)r.h);
+      return r;
+    };
+    P.sff[k].R = split(P.Rk[k]);
+    P.sff[k].cv = split(P.cv[k]);
+    P.sff[k].cp = split(P.cp[k]);
+    P.sff[k].pinf = split(P.pinf[k]);
     if (eos->b[k] != 0.0) P.has_b = 1;
     if (eos->q[k] != 0.0) P.has_q = 1;
   }
