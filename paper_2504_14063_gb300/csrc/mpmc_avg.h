@@ -161,4 +161,30 @@ MPMC_FF bool face_avg_ff(const SpeciesFF* sp, const double* mi, const double* mj
   return true;
 }
 
+// the sound speed at (P, T, Y) and specific volume v: a = c v with
+// c^2 = cp / (T (cp S_2 - S_1^2)), S_q = sum Y_k R_k / (P + Pinf_k)^q.
+// False beyond 2^-60..2^60: the caller takes the FP64 form.
+template <int NS>
+MPMC_FF bool sound_speed_ff(const SpeciesFF* sp, const double* Y, const double p, const double T, const double v,
+                            double& a) {
+  const uint32_t A = 0x7fffffffu, TOP = (1023u + 60u) << 20, BOT = (1023u - 60u) << 20;
+  const uint32_t hp = dhi(p) & A, hT = dhi(T), hv = dhi(v);
+  if (hp >= TOP || hT - BOT >= TOP - BOT || hv - BOT >= TOP - BOT) return false;
+  const ff P0 = ff_of(p), T0 = ff_of(T);
+  ff cp = {0.f, 0.f}, s1 = {0.f, 0.f}, s2 = {0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const ff y = ff_of(Y[k]);
+    const ff r = y.h != 0.f ? ff_rcp(ff_add(P0, sp[k].pinf)) : ff{0.f, 0.f};
+    const ff z = ff_mul(ff_mul(y, sp[k].R), r);
+    cp = ff_add(cp, ff_mul(y, sp[k].cp));
+    s1 = ff_add(s1, z);
+    s2 = ff_add(s2, ff_mul(z, r));
+  }
+  const ff Q = ff_mul(T0, ff_sub(ff_mul(cp, s2), ff_sqr(s1)));
+  if (!(Q.h > 1e-30f && s2.h > 1e-30f && cp.h > 8.67e-19f && cp.h < 1.15e18f)) return false;
+  a = ff_double(ff_mul(ff_sqrt(ff_mul(cp, ff_rcp(Q))), ff_of(v)));
+  return true;
+}
+
 }  // namespace mpmc

@@ -76,6 +76,8 @@ struct KParams {
   // read by the forward FP64 passes (mpmc_fast.cuh)
   WenoEps weno_eps4;  // 4 weno_eps, for the float-float WENO5-Z
   SpeciesFF sff[MAXS];       // Rk, cv, cp, pinf as float-floats
+  double inv_cdi_eps;        // 1 / cdi_eps
+  double cdi_eps_dx, gtol2;  // 1 / cdi_eps, cdi_eps / dx, (4 GTOL dx)^2
 };
 
 // fills P.f32 from the FP64 fields (host)
@@ -209,6 +211,31 @@ __device__ __forceinline__ void load_U(const KParams& P, const double* __restric
 __device__ __forceinline__ double wget(const KParams& P, const double* __restrict__ Wc, int f, CRef r) {
   return Wc[(long long)f * P.wstride + r.idx];
 }
+
+// ---------------------------------------------------------------------------
+// 1/x and 1/sqrt(x) by one third-order step from the hardware's approximation
+// (20 bits: 3 and 5 FP64 operations, an error of an ulp, where the IEEE
+// sequences take 6 to 9).  For finite, normal x; others may give NaN where
+// the division gives infinity or zero.
+__device__ __forceinline__ double drcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  double e = fma(-x, r, 1.0);
+  e = fma(e, e, e);
+  return fma(r, e, r);
+}
+__device__ __forceinline__ double drsqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(e * y, fma(e, 0.375, 0.5), y);
+}
+// |x| in 2^-1000 .. 2^1000, where drcp's result is normal too
+__device__ __forceinline__ bool normal_(double x) {
+  return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 23u < 2000u;
+}
+// a < 0 ? b : c from the sign bit, on the integer pipes
+__device__ __forceinline__ double sel_neg(double a, double b, double c) { return __double2hiint(a) < 0 ? b : c; }
 
 // ---------------------------------------------------------------------------
 // NASG EOS per species (Eq. NASG_EOS)

@@ -68,6 +68,153 @@ __device__ __forceinline__ void recon_lr(const KParams& P, const double* y, doub
   }
 }
 
+// F(S) + s (U*_S - U_S): the HLLC flux on the side S of the contact the
+// face lies on (s = min(0, s_L) for the left side, max(0, s_R) for the right,
+// sS its wave speed, dS = sS - u_S, du = ss - u_S), collected around the two
+// factors
+//   m = u_S + s (f - 1),  w = s f du,  f = dS / (sS - ss),
+// with f - 1 = du / (dS - du) formed without the difference
+template <int NS, int D>
+__device__ __forceinline__ void hllc_one(int d, const State<NS>& S, double s, double dS, double du, double ss,
+                                          double* F) {
+  const double q = du * drcp(dS - du);
+  const double m = fma(s, q, S.u[d]), w = fma(s, q, s) * du;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) F[k] = S.rhoY[k] * m;
+#pragma unroll
+  for (int j = 0; j < D; ++j) F[NS + j] = S.m[j] * m;
+  F[NS + d] += fma(S.rho, w, S.p);
+  F[NS + D] = fma(w, fma(S.rho, ss, S.p * drcp(dS)), fma(S.E, m, S.u[d] * S.p));
+}
+
+template <int NS, int D>
+__device__ __forceinline__ void hllc_flux(int d, const State<NS>& L, const State<NS>& R, double* F) {
+  const double ub = 0.5 * (L.u[d] + R.u[d]), ab = 0.5 * (L.a + R.a);
+  const double sL = fmin(ub - ab, L.u[d] - L.a);
+  const double sR = fmax(ub + ab, R.u[d] + R.a);
+  const double sm = sel_neg(sL, sL, 0.0), sp = sel_neg(sR, 0.0, sR);
+  const double dL = sL - L.u[d], dR = sR - R.u[d];
+  // the contact speed as an increment on u_L (exactly u where P and u are
+  // continuous): ss - u_L = (P_R - P_L - w_R (u_R - u_L)) / (w_L - w_R),
+  // w_S = rho_S (s_S - u_S)
+  const double wL = L.rho * dL, wR = R.rho * dR, Du = R.u[d] - L.u[d];
+  const double duL = fma(-wR, Du, R.p - L.p) * drcp(wL - wR), duR = duL - Du;
+  const double ss = L.u[d] + duL;
+  // only the side of the contact the face lies on is evaluated; sign(0) = 0
+  // takes both with weight 1/2
+  if (positive(ss)) {
+    hllc_one<NS, D>(d, L, sm, dL, duL, ss, F);
+  } else if (negative(ss)) {
+    hllc_one<NS, D>(d, R, sp, dR, duR, ss, F);
+  } else {
+    constexpr int NV = NS + D + 1;
+    double FL[NV], FR[NV];
+    hllc_one<NS, D>(d, L, sm, dL, duL, ss, FL);
+    hllc_one<NS, D>(d, R, sp, dR, duR, ss, FR);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) F[v] = 0.5 * FL[v] + 0.5 * FR[v];
+  }
+}
+
+// the sound speed of eos_forward at (P, T, Y) in FP64, out of line: for
+// states beyond the float-float one's range
+template <int NS>
+__device__ __noinline__ double sound_speed_fp64(const KParams& P, const double* Y, const double p, const double T) {
+  double rho, e, a, al, be;
+  eos_forward<NS>(P, Y, p, T, rho, e, a, al, be);
+  return a;
+}
+
+// face-side state from reconstructed (Y, u, P, T) (steps 4-5 of Sec. 3.1.3).
+// With z_k = Y_k R_k / (P + Pinf_k): v = T sum z_k + sum Y_k b_k and
+// e = T (sum Y_k cv_k + sum Pinf_k z_k) + sum Y_k q_k.  The sound speed only
+// sets HLLC's wave speeds, which act on the two sides' difference: it is
+// float-float (as X and c of the projection).
+template <int NS>
+__device__ __noinline__ void face_state(const KParams& P, const double* Y, const double* u, double p,
+                                                     double T, State<NS>& s) {
+  double vs = 0.0, eb = 0.0, vb = 0.0, eq = 0.0, rg = 0.0;
+  bool have_rg = false;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    if (nonzero(Y[k])) {
+      // ideal-gas species share 1/P
+      double r;
+      if (!nonzero(P.pinf[k])) {
+        if (!have_rg) {
+          rg = drcp(p);
+          have_rg = true;
+        }
+        r = rg;
+      } else {
+        r = drcp(p + P.pinf[k]);
+      }
+      const double z = (Y[k] * P.Rk[k]) * r;
+      vs += z;
+      eb = fma(Y[k], P.cv[k], eb);
+      if (nonzero(P.pinf[k])) eb = fma(P.pinf[k], z, eb);
+      if (P.has_b) vb = fma(Y[k], P.b[k], vb);
+      if (P.has_q) eq = fma(Y[k], P.q[k], eq);
+    }
+  }
+  const double v = fma(T, vs, vb), e = fma(T, eb, eq);
+  s.rho = drcp(v);
+  double ke = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    s.u[d] = u[d];
+    s.m[d] = s.rho * u[d];
+    ke = fma(u[d], u[d], ke);
+  }
+#pragma unroll
+  for (int k = 0; k < NS; ++k) s.rhoY[k] = s.rho * Y[k];
+  s.p = p;
+  s.E = s.rho * fma(0.5, ke, e);
+  if (!sound_speed_ff<NS>(P.sff, Y, p, T, v, s.a)) {
+    double Yc[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) Yc[k] = Y[k];
+    s.a = sound_speed_fp64<NS>(P, Yc, p, T);
+  }
+}
+
+// mass-fraction limiter of Sec. 3.3.1 on one face side (Yc: cell values), as
+// y_limiter with its comparisons on the bits and dd from the sign of Yc - Y
+// (the same values as min(Y, Yc) - Y and max(Y, Yc) - Y)
+template <int NS>
+__device__ __forceinline__ bool limit_Y(double* Y, const double* Yc) {
+  bool active = false;
+#pragma unroll
+  for (int k = 0; k < NS; ++k)
+    if (negative(Y[k])) {
+      Y[k] = 0.0;
+      active = true;
+    }
+  double sum = 0.0;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) sum += Y[k];
+  const double def = 1.0 - sum;
+  // (NaN counts as within the tolerance, as in y_limiter)
+  const unsigned long long db = (unsigned long long)__double_as_longlong(def) & 0x7fffffffffffffffull;
+  if (db > (unsigned long long)__double_as_longlong(NS * YSUM_TOL) && db <= 0x7ff0000000000000ull) {
+    const bool over = __double2hiint(def) < 0;
+    double dd[NS], Sig = 0.0;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      const double t = Yc[k] - Y[k];
+      dd[k] = (__double2hiint(t) < 0) == over ? t : 0.0;
+      Sig += dd[k];
+    }
+    if (nonzero(Sig)) {
+      const double f = normal_(Sig) ? def * drcp(Sig) : def / Sig;
+#pragma unroll
+      for (int k = 0; k < NS; ++k) Y[k] = fma(f, dd[k], Y[k]);
+      active = true;
+    }
+  }
+  return active;
+}
+
 // ---------------------------------------------------------------------------
 // The flux limiter's tests on the FP32 pipe (the FP64 path).  A pseudo-update
 // T = B + s F (B = rk0 U^n + rk1 U^(k)) is first tested on FP32 roundings: a
@@ -77,6 +224,21 @@ __device__ __forceinline__ void recon_lr(const KParams& P, const double* y, doub
 // 1: admissible, 0: not, -1: too close to call (also overflow and NaN).
 constexpr float LIM_MARGIN = 1e-4f;
 constexpr float LIM_TINY = 1e-20f;
+
+// x to FP32 by truncation, on the integer pipes (at most one ulp, 100 times
+// below the margin): below 2^-126 zero, beyond FP32's range NaN (undecided)
+__device__ __forceinline__ float lim_narrow(double x) {
+  const uint32_t H = dhi(x), e = (H >> 20) & 0x7ffu;
+  const uint32_t m = __funnelshift_l(dlo(x), H, 3) & 0x007fffffu;
+  const uint32_t b = (H & 0x80000000u) | ((e - 896u) << 23) | m;
+  return __uint_as_float(e < 897u ? 0u : (e > 1150u ? 0x7fffffffu : b));
+}
+
+// y >= ABSENT (false for NaN) from the bits
+__device__ __forceinline__ bool present_(double y) {
+  const long long b = __double_as_longlong(y);
+  return b >= __double_as_longlong(ABSENT) && b <= 0x7ff0000000000000ll;
+}
 
 // B (value) and M (sum of its terms' magnitudes) of one cell in FP32
 template <int NS, int D>
@@ -90,8 +252,8 @@ __device__ __forceinline__ void limiter_base(const KParams& P, const double* __r
   const long long st = ghost ? P.gstride : P.ncell;
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    float a = rk0 * narrow(un[(long long)v * st]);
-    float b = rk1 != 0.f ? rk1 * narrow(uk[(long long)v * st]) : 0.f;
+    float a = rk0 * lim_narrow(un[(long long)v * st]);
+    float b = rk1 != 0.f ? rk1 * lim_narrow(uk[(long long)v * st]) : 0.f;
     if (v >= NS && v < NS + D && ((r.flip >> (v - NS)) & 1u)) {
       a = -a;
       b = -b;
@@ -177,6 +339,14 @@ __device__ __noinline__ bool admissible_fp64(const KParams& P, const double* Un,
 }
 
 // ---------------------------------------------------------------------------
+// velocity component t of a mapped cell, negated by its sign bit where a wall
+// mirrors it (a multiplication by -1 issues on the FP64 pipe)
+__device__ __forceinline__ double uget(const KParams& P, const double* __restrict__ Wc, int t, CRef r) {
+  const double u = wget(P, Wc, P.wU + t, r);
+  return __hiloint2double(__double2hiint(u) ^ (int)(((r.flip >> t) & 1u) << 31), __double2loint(u));
+}
+
+// ---------------------------------------------------------------------------
 // partial densities of a mapped cell (as load_U)
 template <int NS>
 __device__ __forceinline__ void load_rhoY(const KParams& P, const double* __restrict__ U,
@@ -237,7 +407,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   ci[d] -= 1;  // the cell on the low side of the face
   const double dt = scal[0], Gamma = scal[1];
   // FP32 roundings for the limiter's tests
-  const float rk0f = narrow(rk0), rk1f = narrow(rk1), rk2f = narrow(rk2), dtdx = narrow(dt) * P.f32.inv_dx;
+  const float rk0f = lim_narrow(rk0), rk1f = lim_narrow(rk1), rk2f = lim_narrow(rk2),
+              dtdx = lim_narrow(dt) * P.f32.inv_dx;
 
   CRef cr[6];
 #pragma unroll
@@ -258,8 +429,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     load_rhoY<NS>(P, Uk, Uin, rj, mj);
 #pragma unroll
     for (int t = 0; t < D; ++t) {
-      ui[t] = wget(P, Wc, P.wU + t, ri) * sgn_flip(ri.flip, t);
-      uj[t] = wget(P, Wc, P.wU + t, rj) * sgn_flip(rj.flip, t);
+      ui[t] = uget(P, Wc, t, ri);
+      uj[t] = uget(P, Wc, t, rj);
     }
     if (!face_avg_ff<NS, D>(P.sff, mi, mj, wget(P, Wc, P.wP, ri), wget(P, Wc, P.wP, rj), wget(P, Wc, P.wT, ri),
                             wget(P, Wc, P.wT, rj), ui, uj, X, c, ic)) {
@@ -279,21 +450,22 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     for (int j = 0; j < 6; ++j) {
       const double T = wget(P, Wc, P.wT, cr[j]);
       const double p = wget(P, Wc, P.wP, cr[j]);
-      const double un = wget(P, Wc, P.wU + d, cr[j]) * sgn_flip(cr[j].flip, d);
-      w1[j] = T - X * p;
-      w5[j] = (0.5 * c) * un + 0.5 * p;
-      w6[j] = (-0.5 * c) * un + 0.5 * p;
+      const double un = uget(P, Wc, d, cr[j]);
+      // (twice Appendix A's w5 and w6: the halves are taken once, on the way back)
+      w1[j] = fma(-X, p, T);
+      w5[j] = fma(c, un, p);
+      w6[j] = fma(-c, un, p);
     }
     double w1L, w1R, w5L, w5R, w6L, w6R;
     fast::recon_lr<RC>(P, w1, w1L, w1R);
-    fast::recon_lr<RC>(P, w5, w5L, w5R);
-    fast::recon_lr<RC>(P, w6, w6L, w6R);
-    TL = w1L + X * w5L + X * w6L;
-    TR = w1R + X * w5R + X * w6R;
-    uL[d] = ic * w5L + (-ic) * w6L;
-    uR[d] = ic * w5R + (-ic) * w6R;
-    PL = w5L + w6L;
-    PR = w5R + w6R;
+    fast::recon_lr<RC, true>(P, w5, w5L, w5R);
+    fast::recon_lr<RC, true>(P, w6, w6L, w6R);
+    PL = 0.5 * (w5L + w6L);
+    PR = 0.5 * (w5R + w6R);
+    TL = fma(X, PL, w1L);
+    TR = fma(X, PR, w1R);
+    uL[d] = (0.5 * ic) * (w5L - w6L);
+    uR[d] = (0.5 * ic) * (w5R - w6R);
   }
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
@@ -307,7 +479,7 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     if (t == d) continue;
     double y[6];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) y[j] = wget(P, Wc, P.wU + t, cr[j]) * sgn_flip(cr[j].flip, t);
+    for (int j = 0; j < 6; ++j) y[j] = uget(P, Wc, t, cr[j]);
     fast::recon_lr<RC>(P, y, uL[t], uR[t]);
   }
 
@@ -323,8 +495,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
 
   // interpolation limiters (Sec. 3.3.1)
   if (P.pos_limiter) {
-    if (y_limiter<NS>(YL, Yi)) fl |= F_YLIM_L;
-    if (y_limiter<NS>(YR, Yj)) fl |= F_YLIM_R;
+    if (limit_Y<NS>(YL, Yi)) fl |= F_YLIM_L;
+    if (limit_Y<NS>(YR, Yj)) fl |= F_YLIM_R;
     if (!positive(TL)) { TL = Ti; fl |= F_THETA_T_L; }
     if (!positive(TR)) { TR = Tj; fl |= F_THETA_T_R; }
     bool okL = true, okR = true;
@@ -341,9 +513,9 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   double Fx[NV];
   {
     State<NS> sL, sR;
-    state_from_primitive<NS>(P, YL, uL, PL, TL, sL);
-    state_from_primitive<NS>(P, YR, uR, PR, TR, sR);
-    hllc<NS, D>(d, sL, sR, Fx);
+    face_state<NS>(P, YL, uL, PL, TL, sL);
+    face_state<NS>(P, YR, uR, PR, TR, sR);
+    hllc_flux<NS, D>(d, sL, sR, Fx);
   }
 
   // flux limiter (Sec. 3.3.2): pseudo-updates of both cells, tested on the
@@ -358,7 +530,7 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   auto passes = [&](const double* Ft) {
     float Ff[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) Ff[v] = narrow(Ft[v]);
+    for (int v = 0; v < NV; ++v) Ff[v] = lim_narrow(Ft[v]);
     const int a = admissible_fp32<NS, D>(P, Bi, Mi, Ff, -lamf);
     if (a == 0) return false;
     const int b = admissible_fp32<NS, D>(P, Bj, Mj, Ff, lamf);
@@ -385,8 +557,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     }
 #pragma unroll
     for (int t = 0; t < 3; ++t) {
-      si.u[t] = t < D ? wget(P, Wc, P.wU + t, ri) * sgn_flip(ri.flip, t) : 0.0;
-      sj.u[t] = t < D ? wget(P, Wc, P.wU + t, rj) * sgn_flip(rj.flip, t) : 0.0;
+      si.u[t] = t < D ? uget(P, Wc, t, ri) : 0.0;
+      sj.u[t] = t < D ? uget(P, Wc, t, rj) : 0.0;
       si.m[t] = t < D ? Uki[NS + t] : 0.0;
       sj.m[t] = t < D ? Ukj[NS + t] : 0.0;
     }
@@ -396,7 +568,7 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     sj.E = Ukj[NS + D];
     si.a = wget(P, Wc, P.wA, ri);
     sj.a = wget(P, Wc, P.wA, rj);
-    hllc<NS, D>(d, si, sj, Fx);
+    hllc_flux<NS, D>(d, si, sj, Fx);
     fl |= F_HLLC_FALLBACK;
   }
 
@@ -419,16 +591,17 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
       }
 #pragma unroll
       for (int ph = 0; ph < 2; ++ph) {
-        pres_i[ph] = ypi[ph] >= ABSENT;
-        pres_j[ph] = ypj[ph] >= ABSENT;
+        pres_i[ph] = present_(ypi[ph]);
+        pres_j[ph] = present_(ypj[ph]);
       }
     }
     if ((pres_i[0] || pres_j[0]) && (pres_i[1] || pres_j[1])) {
-      const double ceps = P.cdi_eps;
       const double psi_i = wget(P, Wc, P.wPsi, ri), psi_j = wget(P, Wc, P.wPsi, rj);
-      const double dphi = (wget(P, Wc, P.wPhi0, rj) - wget(P, Wc, P.wPhi0, ri)) * P.inv_dx;
+      const double dphi = wget(P, Wc, P.wPhi0, rj) - wget(P, Wc, P.wPhi0, ri);
+      // the interface normal n_d = d_d psi / |grad psi| from 4 dx grad psi;
+      // zero where |grad psi| < GTOL (the comparisons on the bits)
       double g[3] = {0.0, 0.0, 0.0};
-      g[d] = (psi_j - psi_i) * P.inv_dx;
+      g[d] = 4.0 * (psi_j - psi_i);
 #pragma unroll
       for (int t = 0; t < D; ++t) {
         if (t == d) continue;
@@ -444,20 +617,31 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
         const double pim = wget(P, Wc, P.wPsi, map_cell_dt<d>(P, t, a1[0], a1[1], a1[2]));
         const double pjp = wget(P, Wc, P.wPsi, map_cell_dt<d>(P, t, b0[0], b0[1], b0[2]));
         const double pjm = wget(P, Wc, P.wPsi, map_cell_dt<d>(P, t, b1[0], b1[1], b1[2]));
-        g[t] = 0.5 * ((pip - pim) * (0.5 * P.inv_dx) + (pjp - pjm) * (0.5 * P.inv_dx));
+        g[t] = (pip - pim) + (pjp - pjm);
       }
-      const double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-      const double nd = gn >= GTOL ? g[d] / gn : 0.0;
-      // 1 - tanh^2 as 1 / cosh^2 (no cancellation near the phi_min floor)
-      const double ch = cosh((0.5 * (psi_i + psi_j)) / (2.0 * ceps));
-      const double sech2 = 1.0 / (ch * ch);
-      const double ahat0 = Gamma * (ceps * dphi - 0.25 * (sech2 - P.sharp0) * nd);
+      const double g2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
+      const unsigned long long gb = (unsigned long long)__double_as_longlong(g2),
+                               g_lo = (unsigned long long)__double_as_longlong(P.gtol2),
+                               g_hi = (unsigned long long)__double_as_longlong(1e300);
+      double nd = 0.0;
+      if (gb - g_lo < g_hi - g_lo) nd = g[d] * drsqrt(g2);
+      else if (gb >= g_hi && g2 >= 1e300) nd = g[d] / sqrt(g2);
+      // 1 - tanh^2(x) = sech^2(x) = 4 E / (1 + E)^2, E = exp(-2 |x|), x =
+      // psi / (2 eps): no cancellation near the phi_min floor
+      const double E = exp(-fabs((0.5 * (psi_i + psi_j)) * P.inv_cdi_eps));
+      const double rE = drcp(1.0 + E);
+      // (sech^2 - sharp0) / 4
+      const double sh = fma(E * rE, rE, -0.25 * P.sharp0);
+      const double ahat0 = Gamma * fma(P.cdi_eps_dx, dphi, -sh * nd);
       double Fdi[NV], Rtot = 0.0, hR = 0.0;
 #pragma unroll
       for (int ph = 0; ph < 2; ++ph) {
-        const double ahat = ph == 0 ? ahat0 : -ahat0;
         const bool pi = pres_i[ph], pj = pres_j[ph];
-        auto keep = [&](double a, double b) { return pi && pj ? 0.5 * (a + b) : (pi ? a : (pj ? b : 0.0)); };
+        // the cells' mean, or the value of the one that holds the phase: the
+        // half goes into the velocity
+        const double ah = pi && pj ? 0.5 * ahat0 : ahat0;
+        const double ahat = ph == 0 ? ah : -ah;
+        auto keep = [&](double a, double b) { return pi && pj ? a + b : (pi ? a : (pj ? b : 0.0)); };
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
           if (P.phase[k] != ph) continue;
@@ -470,8 +654,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
       double kb = 0.0;
 #pragma unroll
       for (int t = 0; t < D; ++t) {
-        const double ui = wget(P, Wc, P.wU + t, ri) * sgn_flip(ri.flip, t);
-        const double uj = wget(P, Wc, P.wU + t, rj) * sgn_flip(rj.flip, t);
+        const double ui = uget(P, Wc, t, ri);
+        const double uj = uget(P, Wc, t, rj);
         kb += ui * uj;
         Fdi[NS + t] = 0.5 * (ui + uj) * Rtot;
       }
@@ -497,28 +681,35 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   for (int v = 0; v < NV; ++v) Fnu[v] = 0.0;
   if (P.diffusion) {
     const double rb = 0.5 * (wget(P, Wc, P.wRho, ri) + wget(P, Wc, P.wRho, rj));
-    double Jh = 0.0;
+    // the face enthalpies cp_k T + b_k P + q_k at the two cells' mean P and T;
+    // twice the averages of B and Y, their 1/4 in the common factor
+    const double hrb = -0.25 * P.inv_dx * rb;
+    double Jc = 0.0, Jb = 0.0, Jq = 0.0;
 #pragma unroll
     for (int ph = 0; ph < 2; ++ph) {
-      double Yp = 0.0, S = 0.0, Bf[NS], G[NS];
+      double Yp = 0.0, S = 0.0, Ys[NS], BG[NS];
 #pragma unroll
       for (int k = 0; k < NS; ++k) {
-        Bf[k] = 0.0;
-        G[k] = 0.0;
         if (P.phase[k] != ph) continue;
-        Yp += 0.5 * (Yi[k] + Yj[k]);
-        Bf[k] = 0.5 * (wget(P, Wc, P.wB + k, ri) + wget(P, Wc, P.wB + k, rj));
-        G[k] = (wget(P, Wc, P.wXr + k, rj) - wget(P, Wc, P.wXr + k, ri)) * P.inv_dx;
-        S += Bf[k] * G[k];
+        Ys[k] = Yi[k] + Yj[k];
+        Yp += Ys[k];
+        BG[k] = (wget(P, Wc, P.wB + k, ri) + wget(P, Wc, P.wB + k, rj)) *
+                (wget(P, Wc, P.wXr + k, rj) - wget(P, Wc, P.wXr + k, ri));
+        S += BG[k];
       }
 #pragma unroll
       for (int k = 0; k < NS; ++k) {
         if (P.phase[k] != ph) continue;
-        const double J = -rb * (Yp * Bf[k] * G[k] - 0.5 * (Yi[k] + Yj[k]) * S);
+        const double J = hrb * (Yp * BG[k] - Ys[k] * S);
         Fnu[k] = J;
-        Jh += J * (0.5 * (h_k(P, k, Pi, Ti) + h_k(P, k, Pj, Tj)));
+        Jc = fma(J, P.cp[k], Jc);
+        if (P.has_b) Jb = fma(J, P.b[k], Jb);
+        if (P.has_q) Jq = fma(J, P.q[k], Jq);
       }
     }
+    double Jh = Jc * (0.5 * (Ti + Tj));
+    if (P.has_b) Jh = fma(Jb, 0.5 * (Pi + Pj), Jh);
+    if (P.has_q) Jh += Jq;
     Fnu[NS + D] = Jh;
   }
 
@@ -535,8 +726,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     double ui[3] = {0.0, 0.0, 0.0}, uj[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-      ui[i] = wget(P, Wc, P.wU + i, ri) * sgn_flip(ri.flip, i);
-      uj[i] = wget(P, Wc, P.wU + i, rj) * sgn_flip(rj.flip, i);
+      ui[i] = uget(P, Wc, i, ri);
+      uj[i] = uget(P, Wc, i, rj);
       gu[i][d] = (uj[i] - ui[i]) * P.inv_dx;
     }
 #pragma unroll
@@ -552,10 +743,10 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
       const CRef jp = map_cell_dt<d>(P, t, b0[0], b0[1], b0[2]), jm = map_cell_dt<d>(P, t, b1[0], b1[1], b1[2]);
 #pragma unroll
       for (int i = 0; i < D; ++i) {
-        const double dip = wget(P, Wc, P.wU + i, ip) * sgn_flip(ip.flip, i) -
-                           wget(P, Wc, P.wU + i, im) * sgn_flip(im.flip, i);
-        const double djp = wget(P, Wc, P.wU + i, jp) * sgn_flip(jp.flip, i) -
-                           wget(P, Wc, P.wU + i, jm) * sgn_flip(jm.flip, i);
+        const double dip = uget(P, Wc, i, ip) -
+                           uget(P, Wc, i, im);
+        const double djp = uget(P, Wc, i, jp) -
+                           uget(P, Wc, i, jm);
         gu[i][t] = 0.25 * P.inv_dx * (dip + djp);
       }
     }

@@ -116,6 +116,9 @@ inline int build_params(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_mode
   P.prandtl = m->prandtl;
   P.lambda_liquid = m->lambda_liquid;
   P.cdi_eps = m->cdi_eps > 0.0 ? m->cdi_eps : g->dx;
+  P.inv_cdi_eps = 1.0 / P.cdi_eps;
+  P.cdi_eps_dx = P.cdi_eps * P.inv_dx;
+  P.gtol2 = 16.0 * GTOL * GTOL * P.dx * P.dx;
   P.cdi_gamma = m->cdi_gamma;
   P.phi_min = m->phi_min;
   P.psi_delta = m->psi_delta;
