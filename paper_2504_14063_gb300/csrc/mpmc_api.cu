@@ -217,6 +217,7 @@ extern "C" int mpmc_create(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_m
   }
   c->rec = c->ops;
   if (!mixed) {
+    c->ops.prim = prim_fast(D, ns);
     switch (P.recon) {
       case MPMC_RECON_WENO5JS: c->ops.face = face_fast_weno5js(D, ns); break;
       case MPMC_RECON_TENO5: c->ops.face = face_fast_teno5(D, ns); break;

@@ -76,6 +76,7 @@ struct KParams {
   // read by the forward FP64 passes (mpmc_fast.cuh)
   WenoEps weno_eps4;  // 4 weno_eps, for the float-float WENO5-Z
   SpeciesFF sff[MAXS];       // Rk, cv, cp, pinf as float-floats
+  double iW[MAXS], WSc[MAXS];  // 1 / W, W / Sc
   double inv_cdi_eps;        // 1 / cdi_eps
   double cdi_eps_dx, gtol2;  // 1 / cdi_eps, cdi_eps / dx, (4 GTOL dx)^2
 };
@@ -230,10 +231,18 @@ __device__ __forceinline__ double drsqrt(double x) {
   const double e = fma(-(x * y), y, 1.0);
   return fma(e * y, fma(e, 0.375, 0.5), y);
 }
+// a / b with r = 1 / b to an ulp: the residual's correction, which rounds as
+// the division does (but for ties within 2^-53 of an ulp, and subnormals)
+__device__ __forceinline__ double ddiv(double a, double b, double r) {
+  const double q = a * r;
+  return fma(fma(-b, q, a), r, q);
+}
 // |x| in 2^-1000 .. 2^1000, where drcp's result is normal too
 __device__ __forceinline__ bool normal_(double x) {
   return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 23u < 2000u;
 }
+// a / b to an ulp or two, by the general division where 1 / b is not normal
+__device__ __forceinline__ double qdiv(double a, double b) { return normal_(b) ? a * drcp(b) : a / b; }
 // a < 0 ? b : c from the sign bit, on the integer pipes
 __device__ __forceinline__ double sel_neg(double a, double b, double c) { return __double2hiint(a) < 0 ? b : c; }
 
@@ -1020,6 +1029,21 @@ __device__ __forceinline__ void state_from_primitive(const KParams& P, const dou
   s.E = s.rho * (e + 0.5 * ke);
 }
 
+// every U_k >= -YTOL rho (rho > 0), NaN failing, with the comparisons on the
+// bits: a value without sign against infinity, a negative one's magnitude
+// against YTOL rho's
+template <int NS>
+__device__ __forceinline__ bool rhoY_admissible(const double* U, const double rho) {
+  const unsigned long long lim = (unsigned long long)__double_as_longlong(YTOL * rho);
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(U[k]);
+    ok = ok && (b & 0x7fffffffffffffffull) <= ((b >> 63) ? lim : 0x7ff0000000000000ull);
+  }
+  return ok;
+}
+
 // Eqs. PositivityReqs1/2 on a conserved vector, division free:
 // rhoY_k >= -YTOL rho, rho > 0, 1 - sum rhoY_k b_k > 0,
 // rho E - |m|^2/2 - rho sum rhoY_k q_k > 0
@@ -1036,8 +1060,7 @@ __device__ __forceinline__ bool admissible_bq(const double* b, const double* q, 
   // (without covolumes or reference energies the b and q terms are zero:
   // they are skipped, not evaluated as 1 - 0 and x - 0)
   bool ok = positive(rho) && (!has_b || positive(1.0 - sb));
-#pragma unroll
-  for (int k = 0; k < NS; ++k) ok = ok && (U[k] >= -YTOL * rho);
+  ok = ok && rhoY_admissible<NS>(U, rho);
   double mm = 0.0;
 #pragma unroll
   for (int d = 0; d < D; ++d) mm += U[NS + d] * U[NS + d];

@@ -215,6 +215,323 @@ __device__ __forceinline__ bool limit_Y(double* Y, const double* Yc) {
   return active;
 }
 
+// p-T equilibrium of a cell with r_k = 1 / (P + Pinf_k), for the FP64
+// primitive pass: pt_equilibrium<NS, true> in fewer FP64 operations.  The
+// closed forms keep its order and its rounding (the pressure of a stiff
+// liquid is a small difference); several distinct Pinf: the residual's root
+// from FP32, then a float-float Halley step (to ~2^-46 of the residual's
+// terms), then one Newton step whose residual is FP64; the general iteration
+// where that step is not small against the distance to the nearest pole.
+template <int NS>
+__device__ __forceinline__ int cell_pt(const KParams& P, const double* Y, double e, double v, double& p, double& T,
+                                       double* r) {
+  double Cv = 0.0, q = 0.0, b = 0.0;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    Cv = add_(Cv, mul_(Y[k], P.cv[k]));
+    if (P.has_q) q = add_(q, mul_(Y[k], P.q[k]));
+    if (P.has_b) b = add_(b, mul_(Y[k], P.b[k]));
+  }
+  const double em = P.has_q ? sub_(e, q) : e, vm = P.has_b ? sub_(v, b) : v;
+  int st = ST_OK;
+  if (!positive(em) || !positive(vm)) st = ST_INADMISSIBLE;
+  const double Ep = normal_(vm) ? ddiv(em, vm, drcp(vm)) : em / vm;
+  double pl = -1.0, Rg = 0.0, Rl = 0.0;
+  bool multi = false, gas = false;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    if (positive(Y[k])) {
+      if (positive(P.pinf[k])) {
+        if (negative(pl)) pl = P.pinf[k];
+        else if (bits_of(P.pinf[k]) != bits_of(pl)) multi = true;
+        Rl = add_(Rl, mul_(Y[k], P.Rk[k]));
+      } else {
+        gas = true;
+        Rg = add_(Rg, mul_(Y[k], P.Rk[k]));
+      }
+    }
+  }
+  if (!multi) {
+    double num, den = Cv;
+    if (negative(pl)) {
+      num = mul_(Ep, Rg);
+    } else if (!gas) {
+      num = sub_(sub_(mul_(Ep, Rl), mul_(pl, Cv)), mul_(pl, Rl));
+    } else {
+      const double a2 = sub_(sub_(mul_(Ep, add_(Rg, Rl)), mul_(pl, Cv)), mul_(pl, Rl));
+      const double a3 = mul_(mul_(Ep, pl), Rg);
+      const double sq = sqrt(add_(mul_(a2, a2), mul_(mul_(4.0, Cv), a3)));
+      const double w = add_(fabs(a2), sq);
+      const bool neg = negative(a2);
+      num = neg ? mul_(2.0, a3) : w;
+      den = neg ? w : mul_(2.0, Cv);
+    }
+    p = normal_(den) ? ddiv(num, den, drcp(den)) : num / den;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) r[k] = qdiv(1.0, p + P.pinf[k]);
+  } else {
+    double w[NS], pmin = 1e300;
+    int big = 0;   // the largest |w|'s high word
+    ff wf[NS];
+    const ff Cf = ff_of(Cv);
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      if (positive(Y[k]) && bits_of(P.pinf[k]) < bits_of(pmin)) pmin = P.pinf[k];   // (Pinf >= 0)
+      w[k] = nonzero(Y[k]) ? (Y[k] * P.Rk[k]) * (Ep - P.pinf[k]) : 0.0;
+      wf[k] = ff_of(w[k]);
+      big = max(big, __double2hiint(w[k]) & 0x7fffffff);
+    }
+    const double lo = -pmin;
+    // the quadratic with the liquids merged into one, then the residual, in FP32
+    float x;
+    {
+      float Rgf = 0.f, Rlf = 0.f, wl = 0.f;
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        const float yr = narrow(Y[k]) * P.f32.Rk[k];
+        if (P.f32.pinf[k] > 0.f) {
+          Rlf += yr;
+          wl += yr * P.f32.pinf[k];
+        } else {
+          Rgf += yr;
+        }
+      }
+      const float Ef = narrow(Ep), pe = wl / Rlf;
+      const float a2 = Ef * (Rgf + Rlf) - pe * Cf.h - pe * Rlf;
+      const float sq = sqrtf(fmaxf(a2 * a2 + 4.f * Cf.h * (Ef * pe * Rgf), 0.f));
+      x = a2 >= 0.f ? (a2 + sq) / (2.f * Cf.h) : 2.f * (Ef * pe * Rgf) / (sq - a2);
+    }
+    const float lof = narrow(lo);
+    if (!(x > lof)) x = lof + fmaxf(fabsf(lof), 1.f);
+    x = (float)pt_start_f32<NS>(P, Y, w, Cv, lo, (double)x);
+    // float-float residual, its derivatives in FP32: a Halley step
+    ff xx = {x, 0.f};
+    float df = 0.f, d2 = 0.f;
+    {
+      ff f = {-Cf.h, -Cf.l};
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        if (nonzero(Y[k])) {
+          const ff rk = ff_rcp(ff_add(xx, P.sff[k].pinf));
+          const ff t = ff_mul(wf[k], rk);
+          f = ff_add(f, t);
+          df -= t.h * rk.h;
+          d2 += 2.f * t.h * rk.h * rk.h;
+        }
+      }
+      const float h = 1.f - 0.5f * f.h * d2 / (df * df);
+      xx = ff_add(xx, ff{-f.h / (df * h), 0.f});
+    }
+    p = ff_double(xx);
+    // Newton with the FP64 residual (its derivative in FP32); 1 / (p + Pinf)
+    // follows the step to first order
+    double fd = -Cv;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      r[k] = drcp(p + P.pinf[k]);
+      if (nonzero(Y[k])) fd = fma(w[k], r[k], fd);
+    }
+    const float dxf = -narrow(fd) / df;
+    if (big < (1023 + 100) << 20 && fabsf(dxf) <= 1e-7f * (xx.h - lof) && xx.h < 1e30f) {
+      const double dx = ff_widen(dxf, 1023);
+      p += dx;
+#pragma unroll
+      for (int k = 0; k < NS; ++k) r[k] = fma(-dx * r[k], r[k], r[k]);
+    } else {
+      double Tg;
+      const int s2 = pt_equilibrium<NS>(P, Y, e, v, p, Tg);
+      if (st == ST_OK) st = s2;
+#pragma unroll
+      for (int k = 0; k < NS; ++k) r[k] = 1.0 / (p + P.pinf[k]);
+    }
+  }
+  double den = 0.0;
+#pragma unroll
+  for (int k = 0; k < NS; ++k)
+    if (nonzero(Y[k])) {
+      const double c = Y[k] * P.cv[k];
+      den += nonzero(P.pinf[k]) ? (c * fma(P.gam[k], P.pinf[k], p)) * r[k] : c;
+    }
+  T = normal_(den) ? ddiv(em, den, drcp(den)) : em / den;
+  return st;
+}
+
+// ---------------------------------------------------------------------------
+// the forward FP64 primitive pass: mpmc_kernels.cuh's k_prim with its divisions
+// taken from shared reciprocals and the several-liquid p-T solve's iterations
+// on the FP32 pipe (cell_pt)
+template <int NS, int D>
+__global__ void __launch_bounds__(CELL_THREADS)
+    k_prim(const KParams P, const double* __restrict__ U, const double* __restrict__ Uin, double* __restrict__ Wc,
+           unsigned long long* __restrict__ red, int* __restrict__ status) {
+  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  double smax = 0.0, gmax = 0.0;
+  if (c < P.ncell + P.nextra) {
+    constexpr int NV = NS + D + 1;
+    double Uc[NV];
+    if (c >= P.ncell) {
+      // the inflow state or a characteristic ghost, from U's ghost buffer
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Uc[v] = Uin[(long long)v * P.gstride + (c - P.ncell)];
+    } else {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Uc[v] = U[(long long)v * P.ncell + c];
+    }
+    const long long ws = P.wstride;
+    // decode in the oracle's order and rounding, the divisions by rho from one
+    // reciprocal
+    double rho = 0.0, Y[NS], u[3], e, irho, ke = 0.0;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) rho = add_(rho, Uc[k]);
+    if (normal_(rho)) {
+      irho = drcp(rho);
+      irho = fma(fma(-rho, irho, 1.0), irho, irho);
+#pragma unroll
+      for (int k = 0; k < NS; ++k) Y[k] = ddiv(Uc[k], rho, irho);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        u[d] = d < D ? ddiv(Uc[NS + d], rho, irho) : 0.0;
+        if (d < D) ke = add_(ke, mul_(u[d], u[d]));
+      }
+      e = sub_(ddiv(Uc[NS + D], rho, irho), mul_(0.5, ke));
+    } else {
+      decode<NS, D>(Uc, rho, Y, u, e, irho);
+    }
+    int st = positive(rho) ? ST_OK : ST_INADMISSIBLE;
+    if (!rhoY_admissible<NS>(Uc, rho)) st = ST_INADMISSIBLE;
+    double p, T, r[NS];
+    const int st2 = cell_pt<NS>(P, Y, e, irho, p, T, r);
+    if (st == ST_OK) st = st2;
+    // sound speed: a = c v, c^2 = cp / (T (cp S_2 - S_1^2)), S_q = sum Y_k R_k r_k^q
+    double a, z[NS];
+    {
+      double cp = 0.0, s1 = 0.0, s2 = 0.0;
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        z[k] = nonzero(Y[k]) ? (Y[k] * P.Rk[k]) * r[k] : 0.0;
+        cp = fma(Y[k], P.cp[k], cp);
+        s1 += z[k];
+        if (nonzero(Y[k])) s2 = fma(z[k], r[k], s2);
+      }
+      a = (cp * irho) * drsqrt(cp * (T * fma(cp, s2, -s1 * s1)));
+    }
+    Wc[P.wT * ws + c] = T;
+    Wc[P.wP * ws + c] = p;
+    Wc[P.wRho * ws + c] = rho;
+    Wc[P.wA * ws + c] = a;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) Wc[(P.wY + k) * ws + c] = Y[k];
+#pragma unroll
+    for (int d = 0; d < D; ++d) Wc[(P.wU + d) * ws + c] = u[d];
+
+    double mu = 0.0, lam = 0.0;
+    if (P.cdi || P.diffusion || P.viscous) {
+      double phi[2], Yp[2];
+      const double rT = rho * T;
+#pragma unroll
+      for (int ph = 0; ph < 2; ++ph) {
+        // phi_p = sum U_k v_k = rho T sum z_k + sum U_k b_k, h_p rho_p phi_p = sum U_k h_k
+        double f = 0.0, hr = 0.0, yp = 0.0, hb = 0.0, hq = 0.0;
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+          if (P.phase[k] == ph) {
+            yp += Y[k];
+            f += z[k];
+            hr = fma(Uc[k], P.cp[k], hr);
+            if (P.has_b) hb = fma(Uc[k], P.b[k], hb);
+            if (P.has_q) hq = fma(Uc[k], P.q[k], hq);
+          }
+        f = fma(rT, f, hb);
+        hr *= T;
+        if (P.has_b) hr = fma(p, hb, hr);
+        if (P.has_q) hr += hq;
+        phi[ph] = f;
+        Yp[ph] = yp;
+        if (P.cdi) {
+          const bool present = yp >= ABSENT;
+          const double rf = qdiv(1.0, f);
+          Wc[(P.wHrho + ph) * ws + c] = present ? hr * rf : 0.0;
+#pragma unroll
+          for (int k = 0; k < NS; ++k)
+            if (P.phase[k] == ph) Wc[(P.wYrho + k) * ws + c] = present ? Uc[k] * rf : 0.0;
+        }
+      }
+      if (P.cdi) {
+        Wc[P.wPhi0 * ws + c] = phi[0];
+        Wc[P.wPsi * ws + c] = P.cdi_eps * log(qdiv(phi[0] + P.psi_delta, phi[1] + P.psi_delta));
+      }
+      // phase viscosities: liquid constant, gas by Wilke's rule
+      double mup[2] = {P.mu_liquid, 0.0};
+      if (P.diffusion || P.viscous) {
+        double num = 0.0;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+          if (P.phase[i] != 1) continue;
+          double den = 0.0;
+#pragma unroll
+          for (int j = 0; j < NS; ++j)
+            if (P.phase[j] == 1) den = fma(Y[j], P.wilke[i][j], den);
+          if (positive(den)) num += qdiv(Y[i] * P.mu[i], den);
+        }
+        mup[1] = Yp[1] >= ABSENT ? num : 0.0;
+        mu = phi[0] * mup[0] + phi[1] * mup[1];
+      }
+      if (P.viscous) {
+        // heat conductivity: liquid constant, gas (mu_g / Pr) sum (Y^c/Y_g) Cp^c
+        double cpY = 0.0;
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+          if (P.phase[k] == 1) cpY += Y[k] * P.cp[k];
+        const double lam_g = Yp[1] >= ABSENT ? mup[1] / P.prandtl * (cpY / Yp[1]) : 0.0;
+        lam = phi[0] * P.lambda_liquid + phi[1] * lam_g;
+        Wc[P.wMu * ws + c] = mu;
+        Wc[P.wLam * ws + c] = lam;
+      }
+      if (P.diffusion) {
+        // X^c/X_p = (Y^c/W^c) / sY, sY = sum_p Y/W;
+        // W^c D^c / W_p = (W^c/Sc^c) (sY/Y_p) mu_p (phi_p/Y_p) / rho
+#pragma unroll
+        for (int ph = 0; ph < 2; ++ph) {
+          double sY = 0.0, yw[NS];
+#pragma unroll
+          for (int j = 0; j < NS; ++j)
+            if (P.phase[j] == ph) {
+              yw[j] = Y[j] * P.iW[j];
+              sY += yw[j];
+            }
+          const bool present = Yp[ph] >= ABSENT && sY >= ABSENT;
+          const double ry = qdiv(1.0, Yp[ph]), rs = qdiv(1.0, sY);
+          const double Bp = (sY * ry) * ((mup[ph] * irho) * (phi[ph] * ry));
+#pragma unroll
+          for (int k = 0; k < NS; ++k) {
+            if (P.phase[k] != ph) continue;
+            Wc[(P.wXr + k) * ws + c] = present ? yw[k] * rs : 0.0;
+            Wc[(P.wB + k) * ws + c] = present ? P.WSc[k] * Bp : 0.0;
+          }
+        }
+      }
+    }
+    if (st != ST_OK) atomicMax(status, st);
+    if (c < P.ncell) {
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const double ud = fabs(u[d]);
+        smax = fmax(smax, (ud + a) * P.inv_dx);
+        gmax = fmax(gmax, ud);
+      }
+      if (P.diffusion || P.viscous) smax = fmax(smax, 4.0 * mu * irho * (P.inv_dx * P.inv_dx));
+      if (P.viscous) {
+        // conduction limit with the thermal diffusivity lambda / (rho cv)
+        double cv = 0.0;
+#pragma unroll
+        for (int k = 0; k < NS; ++k) cv += Y[k] * P.cv[k];
+        smax = fmax(smax, 4.0 * lam / (rho * cv) * (P.inv_dx * P.inv_dx));
+      }
+    }
+  }
+  if (red) block_max2(smax, gmax, red);
+}
+
 // ---------------------------------------------------------------------------
 // The flux limiter's tests on the FP32 pipe (the FP64 path).  A pseudo-update
 // T = B + s F (B = rk0 U^n + rk1 U^(k)) is first tested on FP32 roundings: a
@@ -787,6 +1104,12 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     if (fl & (F_YLIM_L | F_YLIM_R)) atomicAdd(stats + 5, 1ull);
     if (fl & F_DIFF_DROPPED) atomicAdd(stats + 6, 1ull);
   }
+}
+
+template <int NS, int D>
+void prim(const KParams& P, cudaStream_t s, const double* U, const double* Uin, double* Wc, unsigned long long* red,
+          int* status) {
+  fast::k_prim<NS, D><<<nblocks(P.ncell + P.nextra, CELL_THREADS), CELL_THREADS, 0, s>>>(P, U, Uin, Wc, red, status);
 }
 
 // the forward FP64 face pass of one direction with interpolation RC

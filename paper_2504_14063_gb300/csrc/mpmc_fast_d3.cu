@@ -1,4 +1,4 @@
-// Forward FP64 face-pass instantiations (WENO5-Z) for dimension 3, species counts 1..4.
+// Forward FP64 primitive- and face-pass instantiations (WENO5-Z) for dimension 3, species counts 1..4.
 #include "mpmc_fast.cuh"
 
 namespace mpmc {
@@ -9,6 +9,16 @@ FaceFn face_fast_d3(int ns) {
     case 2: return &fast::FaceImpl<2, 3, RC_WENO5Z>::face;
     case 3: return &fast::FaceImpl<3, 3, RC_WENO5Z>::face;
     case 4: return &fast::FaceImpl<4, 3, RC_WENO5Z>::face;
+    default: return nullptr;
+  }
+}
+
+PrimFn prim_fast_d3(int ns) {
+  switch (ns) {
+    case 1: return &fast::prim<1, 3>;
+    case 2: return &fast::prim<2, 3>;
+    case 3: return &fast::prim<3, 3>;
+    case 4: return &fast::prim<4, 3>;
     default: return nullptr;
   }
 }

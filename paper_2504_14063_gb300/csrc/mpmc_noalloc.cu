@@ -97,6 +97,7 @@ extern "C" int mpmc_rhs_noalloc(const mpmc_grid* grid, const mpmc_eos* eos, cons
   // is and not cleared: the final check below then only sees this call's
   if (cudaPeekAtLastError() != cudaSuccess) return MPMC_CUDA_ERROR;
   Ops ops = P.dim == 1 ? ops_fp64_d1(P.ns) : (P.dim == 2 ? ops_fp64_d2(P.ns) : ops_fp64_d3(P.ns));
+  ops.prim = prim_fast(P.dim, P.ns);
   ops.face = face_fast_weno5z(P.dim, P.ns);
   if (!ops.face) return MPMC_INVALID_ARG;
   void* base = nullptr;

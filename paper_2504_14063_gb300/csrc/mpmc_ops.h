@@ -42,15 +42,19 @@ struct AdjOps {
 };
 
 using FaceFn = decltype(Ops::face);
+using PrimFn = decltype(Ops::prim);
 // FP64 face passes with Sec. 4.1's other ENO-type interpolations, for
 // (dimension, species count), null if none: defined in
 // mpmc_recon_{weno5js,teno5,teno6}.cu
 FaceFn face_fp64_weno5js(int dim, int ns);
 FaceFn face_fp64_teno5(int dim, int ns);
 FaceFn face_fp64_teno6(int dim, int ns);
-// forward FP64 face passes (float-float interpolation weights), the ones that
+// forward FP64 primitive and face passes (parts in float-float), the ones that
 // steps and right-hand sides run: mpmc_fast_d{1,2,3}.cu,
 // mpmc_fast_{weno5js,teno5,teno6}.cu
+PrimFn prim_fast_d1(int ns);
+PrimFn prim_fast_d2(int ns);
+PrimFn prim_fast_d3(int ns);
 FaceFn face_fast_d1(int ns);
 FaceFn face_fast_d2(int ns);
 FaceFn face_fast_d3(int ns);
@@ -69,6 +73,9 @@ AdjFaceFn adj_face_weno5js(int dim, int ns);
 AdjFaceFn adj_face_teno5(int dim, int ns);
 AdjFaceFn adj_face_teno6(int dim, int ns);
 
+inline PrimFn prim_fast(int dim, int ns) {
+  return dim == 1 ? prim_fast_d1(ns) : (dim == 2 ? prim_fast_d2(ns) : prim_fast_d3(ns));
+}
 inline FaceFn face_fast_weno5z(int dim, int ns) {
   return dim == 1 ? face_fast_d1(ns) : (dim == 2 ? face_fast_d2(ns) : face_fast_d3(ns));
 }

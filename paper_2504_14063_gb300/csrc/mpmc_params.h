@@ -73,6 +73,8 @@ inline int build_params(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_mode
     P.b[k] = eos->b[k];
     P.pinf[k] = eos->pinf[k];
     P.W[k] = eos->W[k];
+    P.iW[k] = 1.0 / eos->W[k];
+    P.WSc[k] = eos->W[k] / eos->Sc[k];
     P.mu[k] = eos->mu[k];
     P.Sc[k] = eos->Sc[k];
     P.Rk[k] = (eos->gamma[k] - 1.0) * eos->cv[k];
