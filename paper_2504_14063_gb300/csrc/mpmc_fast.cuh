@@ -24,11 +24,12 @@ namespace fast {
 // the FP64 form of both sides, for stencils outside the range of the
 // float-float one (differences that are not finite or beyond 2^900); out of
 // line, so that it costs the callers no registers
-static __device__ __noinline__ double2 weno5z_lr_fp64(double w0, double w1, double w2, double w3, double w4,
-                                                      double w5, double eps) {
+template <int RC>
+__device__ __noinline__ double2 eno_lr_fp64(double w0, double w1, double w2, double w3, double w4, double w5,
+                                            double eps) {
   const double w[6] = {w0, w1, w2, w3, w4, w5};
   double L, R;
-  mpmc::recon_lr<RC_WENO5Z>(w, eps, L, R);
+  mpmc::recon_lr<RC>(w, eps, L, R);
   return make_double2(L, R);
 }
 
@@ -38,34 +39,35 @@ static __device__ __noinline__ double2 weno5z_lr_fp64(double w0, double w1, doub
 // long as it issued them (droplet field 128^3, faces of a step: 46.4 ms
 // inlined, 39.3 ms with this function called, 33.8 ms with the face states
 // and the limiter's tests called too).
-static __device__ __noinline__ double2 weno5z_lr(double w0, double w1, double w2, double w3, double w4, double w5, float eh, float el,
-                              int ee) {
+// two: twice the method's field (eps, compared with its square, then counts
+// four times).  (In the FP64 form of TENO and WENO5-JS, whose eps is fixed,
+// the doubled field is halved and its values doubled.)
+template <int RC>
+__device__ __noinline__ double2 eno_lr(double w0, double w1, double w2, double w3, double w4, double w5, float eh,
+                                       float el, int ee, int two) {
   const double w[6] = {w0, w1, w2, w3, w4, w5};
+  WenoEps e = {eh, el, ee + 2 * two};
+  if constexpr (RC == RC_WENO5JS) e = js_eps4(2 * two);
+  if constexpr (RC == RC_TENO5 || RC == RC_TENO6) e = teno_eps4(2 * two);
   double L, R;
-  if (weno5z_lr_ff(w, WenoEps{eh, el, ee}, L, R)) return make_double2(L, R);
-  return weno5z_lr_fp64(w0, w1, w2, w3, w4, w5, 0.25 * scalbn((double)eh + (double)el, ee));
+  if (eno_lr_ff<RC>(w, e, L, R)) return make_double2(L, R);
+  const double h = two ? 0.5 : 1.0, g = two ? 2.0 : 1.0;
+  double2 v = eno_lr_fp64<RC>(h * w0, h * w1, h * w2, h * w3, h * w4, h * w5,
+                              0.25 * scalbn((double)eh + (double)el, ee));
+  v.x *= g;
+  v.y *= g;
+  return v;
 }
 
 // both face values of one field from the cells y[0..5] = i-2..i+3 around
-// the face i+1/2; WENO5-Z in float-float (mpmc_ff.h).  TWICE: the field is
-// twice the method's (eps, compared with its square, then counts four times).
+// the face i+1/2, in float-float (mpmc_ff.h).  TWICE: the field is twice the
+// method's.
 template <int RC, bool TWICE = false>
 __device__ __forceinline__ void recon_lr(const KParams& P, const double* y, double& L, double& R) {
-  if constexpr (RC == RC_WENO5Z) {
-    const double2 v = weno5z_lr(y[0], y[1], y[2], y[3], y[4], y[5], P.weno_eps4.h, P.weno_eps4.l,
-                                P.weno_eps4.e + (TWICE ? 2 : 0));
-    L = v.x;
-    R = v.y;
-  } else if constexpr (TWICE) {
-    double h[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) h[j] = 0.5 * y[j];
-    mpmc::recon_lr<RC>(h, P.weno_eps, L, R);
-    L *= 2.0;
-    R *= 2.0;
-  } else {
-    mpmc::recon_lr<RC>(y, P.weno_eps, L, R);
-  }
+  const double2 v = eno_lr<RC>(y[0], y[1], y[2], y[3], y[4], y[5], P.weno_eps4.h, P.weno_eps4.l, P.weno_eps4.e,
+                               TWICE ? 1 : 0);
+  L = v.x;
+  R = v.y;
 }
 
 // F(S) + s (U*_S - U_S): the HLLC flux on the side S of the contact the
