@@ -239,7 +239,7 @@ extern "C" int mpmc_create(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_m
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
     c->nface[d] = nf;
     c->nface_total += nf;
-    rc = alloc(c, (void**)&c->F[d], (size_t)P.nv * nf * sizeof(double));
+    rc = alloc(c, (void**)&c->F[d], (size_t)P.nv * nf * (mixed ? sizeof(float) : sizeof(double)));
   }
   if (!rc && mixed) {
     // FP32 copy of U^n for the mixed path's limiter (read by its face kernel)

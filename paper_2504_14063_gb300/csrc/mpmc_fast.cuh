@@ -535,24 +535,6 @@ __global__ void __launch_bounds__(CELL_THREADS)
 }
 
 // ---------------------------------------------------------------------------
-// The flux limiter's tests on the FP32 pipe (the FP64 path).  A pseudo-update
-// T = B + s F (B = rk0 U^n + rk1 U^(k)) is first tested on FP32 roundings: a
-// test is decided there only when its value clears LIM_MARGIN times the
-// magnitudes of its terms, 100 times what FP32 rounding can move it, and
-// when it is far from FP32 underflow; so a decision is the FP64 test's own.
-// 1: admissible, 0: not, -1: too close to call (also overflow and NaN).
-constexpr float LIM_MARGIN = 1e-4f;
-constexpr float LIM_TINY = 1e-20f;
-
-// x to FP32 by truncation, on the integer pipes (at most one ulp, 100 times
-// below the margin): below 2^-126 zero, beyond FP32's range NaN (undecided)
-__device__ __forceinline__ float lim_narrow(double x) {
-  const uint32_t H = dhi(x), e = (H >> 20) & 0x7ffu;
-  const uint32_t m = __funnelshift_l(dlo(x), H, 3) & 0x007fffffu;
-  const uint32_t b = (H & 0x80000000u) | ((e - 896u) << 23) | m;
-  return __uint_as_float(e < 897u ? 0u : (e > 1150u ? 0x7fffffffu : b));
-}
-
 // y >= ABSENT (false for NaN) from the bits
 __device__ __forceinline__ bool present_(double y) {
   const long long b = __double_as_longlong(y);
@@ -593,52 +575,8 @@ __device__ __noinline__ int admissible_fp32(const KParams& P, const float* B, co
     T[v] = B[v] + f;
     G[v] = M[v] + fabsf(f);
   }
-  bool undecided = false;
-  auto test = [&](float val, float mag) {
-    if (val > LIM_MARGIN * mag) return true;
-    if (!(val < -LIM_MARGIN * mag)) undecided = true;
-    return false;
-  };
-  float rho = 0.f, Grho = 0.f;
-#pragma unroll
-  for (int k = 0; k < NS; ++k) {
-    rho += T[k];
-    Grho += G[k];
-  }
-  bool ok = test(rho, Grho);
-  float sq = 0.f, Gsq = 0.f;
-  if (P.has_b) {
-    float sb = 0.f, Gsb = 1.f;
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      sb += T[k] * P.f32.b[k];
-      Gsb += G[k] * fabsf(P.f32.b[k]);
-    }
-    ok = test(1.f - sb, Gsb) && ok;
-  }
-  if (P.has_q) {
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      sq += T[k] * P.f32.q[k];
-      Gsq += G[k] * fabsf(P.f32.q[k]);
-    }
-  }
-  const float yt = (float)YTOL;
-#pragma unroll
-  for (int k = 0; k < NS; ++k) ok = test(T[k] + yt * rho, G[k] + yt * Grho) && ok;
-  float mm = 0.f, Gmm = 0.f;
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    mm += T[NS + d] * T[NS + d];
-    Gmm += G[NS + d] * G[NS + d];
-  }
-  const float Ge = Grho * G[NS + D] + 0.5f * Gmm + Grho * Gsq;
-  ok = test(rho * T[NS + D] - 0.5f * mm - rho * sq, Ge) && ok;
-  // terms near FP32's underflow are not judged by their FP32 magnitudes
-  if (!(Grho > LIM_TINY && Ge > LIM_TINY && fabsf(s) > LIM_TINY)) return -1;
-  if (ok) return 1;
-  // a test decided "no" makes the state inadmissible whatever the others say
-  return undecided ? -1 : 0;
+  const int a = admissible_margin<NS, D>(P, T, G);
+  return fabsf(s) > LIM_TINY ? a : -1;
 }
 
 // the FP64 test of T = rk0 U^n + rk1 U^(k) + s F, for a flux that the FP32

@@ -672,7 +672,7 @@ template <int NS, int D, int DIR, int RC>
 __global__ void __launch_bounds__(FACE_THREADS, 5)
     k_face(const KParams P, const float* __restrict__ Wc, const double* __restrict__ Un,
            const double* __restrict__ Uk, const double* __restrict__ Uin, const double* __restrict__ scal,
-           const double rk0, const double rk1, const double rk2, double* __restrict__ F,
+           const double rk0, const double rk1, const double rk2, float* __restrict__ F,
            uint32_t* __restrict__ flags, unsigned long long* __restrict__ stats) {
   constexpr int NV = NS + D + 1;
   constexpr int d = DIR;
@@ -1050,10 +1050,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 5)
     }
   }
 
-  // stored widened to FP64 (exact): the update then takes every flux with
-  // the same FP64 value in its two cells, and the widening happens once per
-  // face, here, where the FP64 pipe is otherwise idle
-  for (int v = 0; v < NV; ++v) F[(long long)v * nf + fid] = (double)Fx[v];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) F[(long long)v * nf + fid] = Fx[v];
   if (flags) flags[fid] = fl;
   if (stats && fl) {
     if (fl & F_HLLC_FALLBACK) atomicAdd(stats + 1, 1ull);
@@ -1065,11 +1063,12 @@ __global__ void __launch_bounds__(FACE_THREADS, 5)
   }
 }
 
-// divergence and RK combination in FP64 (the FP64 path's, on the widened fluxes)
+// divergence of the FP32 fluxes (their differences in float-float) and RK
+// combination in FP64
 template <int NS, int D>
 __global__ void __launch_bounds__(CELL_THREADS)
     k_update(const KParams P, const double* __restrict__ Un, const double* __restrict__ Uk,
-             const double* __restrict__ F0, const double* __restrict__ F1, const double* __restrict__ F2,
+             const float* __restrict__ F0, const float* __restrict__ F1, const float* __restrict__ F2,
              const double* __restrict__ scal, const double rk0, const double rk1, const double rk2,
              double* __restrict__ Uout, double* __restrict__ dUdt, int* __restrict__ status) {
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1089,13 +1088,14 @@ struct FaceImpl {
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
     const unsigned nb = nblocks(nf, FACE_THREADS);
     const float* W = reinterpret_cast<const float*>(Wc);
+    float* Ff = reinterpret_cast<float*>(F);   // the mixed path's fluxes are FP32
     if (d == 0)
-      k_face<NS, D, 0, RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, F, flags, stats);
+      k_face<NS, D, 0, RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff, flags, stats);
     else if (d == 1)
-      k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+      k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff,
                                                                      flags, stats);
     else
-      k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+      k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff,
                                                                      flags, stats);
   }
 };
@@ -1135,8 +1135,10 @@ struct Impl {
   static void update(const KParams& P, cudaStream_t s, const double* Un, const double* Uk, double* const* F,
                      const double* scal, double rk0, double rk1, double rk2, double* Uout, double* dUdt,
                      int* status) {
-    k_update<NS, D><<<nblocks(P.ncell, CELL_THREADS), CELL_THREADS, 0, s>>>(
-        P, Un, Uk, F[0], D > 1 ? F[1] : F[0], D > 2 ? F[2] : F[0], scal, rk0, rk1, rk2, Uout, dUdt, status);
+    const float* Ff[3];
+    for (int d = 0; d < 3; ++d) Ff[d] = reinterpret_cast<const float*>(F[d < D ? d : 0]);
+    k_update<NS, D><<<nblocks(P.ncell, CELL_THREADS), CELL_THREADS, 0, s>>>(P, Un, Uk, Ff[0], Ff[1], Ff[2], scal,
+                                                                            rk0, rk1, rk2, Uout, dUdt, status);
   }
 };
 

@@ -65,6 +65,33 @@ MPMC_HD2 uint64_t bits_of(double x) {
 #endif
 }
 
+// FP32 -> FP64, exactly, on the integer pipes, of a normal number or zero
+MPMC_HD2 uint32_t bits_f(float f) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(f);
+#else
+  uint32_t u;
+  std::memcpy(&u, &f, 4);
+  return u;
+#endif
+}
+MPMC_HD2 bool widens(float f) {
+  const uint32_t m = bits_f(f) & 0x7fffffffu;
+  return m - 0x00800000u < 0x7f000000u || m == 0u;
+}
+MPMC_HD2 double widen(float f) {
+  const uint32_t b = bits_f(f), m = b & 0x7fffffffu;
+  const uint32_t hi = (b & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u);
+#ifdef __CUDA_ARCH__
+  return __hiloint2double((int)hi, (int)(b << 29));
+#else
+  const uint64_t u = ((uint64_t)hi << 32) | (uint32_t)(b << 29);
+  double x;
+  std::memcpy(&x, &u, 8);
+  return x;
+#endif
+}
+
 // y != 0, y > 0 and y < 0 from the bits, on the integer pipes (an FP64 comparison
 // issues on the FP64 pipe, which binds the FP64 kernels); the same results
 // as the comparisons for every input: +-0 is zero, NaN is nonzero and not

@@ -1,18 +1,68 @@
 // Divergence of the face fluxes (Eq. DiscreteGoverningEquations) and the
-// SSP-RK combination (Eq. SSPRK3) of one cell, from FP64 face fluxes
-// F_d[v][face]; shared by the FP64 and mixed-precision update kernels (the
-// mixed face kernel stores its FP32 fluxes widened to FP64, exactly, so that
-// every flux enters its two cells with the same FP64 value and the sum over
-// cells telescopes to FP64 rounding).
+// SSP-RK combination (Eq. SSPRK3) of one cell, from face fluxes F_d[v][face]
+// of type FT: double, or float on the mixed path (every flux enters its two
+// cells with the same value, so that the sum over cells telescopes to the
+// rounding of the combination).
 #pragma once
 #include "mpmc_device.cuh"
 
 namespace mpmc {
 
-template <int NS, int D>
+// fs[v] = sum_d (F_d[m_d] - F_d[p_d]) of every component
+template <int NV, int D>
+__device__ __forceinline__ void flux_sums(const double* const* Fd, const long long* nf, const long long* fm,
+                                          const long long* fp, double* fs) {
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    fs[v] = Fd[0][(long long)v * nf[0] + fm[0]] - Fd[0][(long long)v * nf[0] + fp[0]];
+#pragma unroll
+    for (int d = 1; d < D; ++d) fs[v] += Fd[d][(long long)v * nf[d] + fm[d]] - Fd[d][(long long)v * nf[d] + fp[d]];
+  }
+}
+
+// the same of FP32 fluxes: the differences exactly as float-floats, their sum
+// to 2^-47 of the largest, on the FP32 pipe.  (FP64 differences and sums, on
+// fluxes widened by the face pass, were 5 of the update's 8 FP64 operations
+// per component in 3D, and twice the flux traffic.)  Sums beyond FP32's normal
+// range take FP64, once all are formed: a branch per component would keep the
+// next one's loads back.
+template <int NV, int D>
+__device__ __forceinline__ void flux_sums(const float* const* Fd, const long long* nf, const long long* fm,
+                                          const long long* fp, double* fs) {
+  float a[NV][D], b[NV][D];
+#pragma unroll
+  for (int v = 0; v < NV; ++v)
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      a[v][d] = Fd[d][(long long)v * nf[d] + fm[d]];
+      b[v][d] = Fd[d][(long long)v * nf[d] + fp[d]];
+    }
+  bool general = false;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    ff s = ff_two(a[v][0], -b[v][0]);
+#pragma unroll
+    for (int d = 1; d < D; ++d) s = ff_add(s, ff_two(a[v][d], -b[v][d]));
+    general = general || !widens(s.h) || !widens(s.l);
+    fs[v] = widen(s.h) + widen(s.l);
+  }
+  if (general) {
+#pragma unroll 1
+    for (int v = 0; v < NV; ++v) {
+      double f = (double)Fd[0][(long long)v * nf[0] + fm[0]] - (double)Fd[0][(long long)v * nf[0] + fp[0]];
+      for (int d = 1; d < D; ++d)
+        f += (double)Fd[d][(long long)v * nf[d] + fm[d]] - (double)Fd[d][(long long)v * nf[d] + fp[d]];
+#pragma unroll
+      for (int w = 0; w < NV; ++w)
+        if (w == v) fs[w] = f;
+    }
+  }
+}
+
+template <int NS, int D, typename FT>
 __device__ __forceinline__ void update_cell(const KParams& P, const long long c, const double* __restrict__ Un,
-                                            const double* __restrict__ Uk, const double* __restrict__ F0,
-                                            const double* __restrict__ F1, const double* __restrict__ F2,
+                                            const double* __restrict__ Uk, const FT* __restrict__ F0,
+                                            const FT* __restrict__ F1, const FT* __restrict__ F2,
                                             const double* __restrict__ scal, const double rk0, const double rk1,
                                             const double rk2, double* __restrict__ Uout, double* __restrict__ dUdt,
                                             int* __restrict__ status) {
@@ -21,7 +71,7 @@ __device__ __forceinline__ void update_cell(const KParams& P, const long long c,
   int ijk[3];
   unflatten(c, n0, n1, ijk);
   const int i = ijk[0], j = ijk[1], k = ijk[2];
-  const double* Fd[3] = {F0, F1, F2};
+  const FT* Fd[3] = {F0, F1, F2};
   long long fm[3], fp[3], nf[3];
 #pragma unroll
   for (int d = 0; d < D; ++d) {
@@ -38,27 +88,34 @@ __device__ __forceinline__ void update_cell(const KParams& P, const long long c,
   // the coefficient tests, once per thread as integers (FP64 comparisons
   // issue on the FP64 pipe, and would otherwise be repeated per variable)
   const int keep = dt == 0.0, use_k = rk1 != 0.0, use_n = rk0 != 0.0;
-  double Uo[NV];
+  // (all loads before the first use: a conditional load per component would
+  // wait for the one before)
+  double Uo[NV], fs[NV], un[NV], uk[NV];
+  if (use_n) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) un[v] = Un[(long long)v * P.ncell + c];
+  }
+  if (use_k | keep) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) uk[v] = Uk[(long long)v * P.ncell + c];
+  }
+  flux_sums<NV, D>(Fd, nf, fm, fp, fs);
+  if (dUdt) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) dUdt[(long long)v * P.ncell + c] = fs[v] * P.inv_dx;
+  }
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    double fs = Fd[0][(long long)v * nf[0] + fm[0]] - Fd[0][(long long)v * nf[0] + fp[0]];
-#pragma unroll
-    for (int d = 1; d < D; ++d) fs += Fd[d][(long long)v * nf[d] + fm[d]] - Fd[d][(long long)v * nf[d] + fp[d]];
-    if (dUdt) dUdt[(long long)v * P.ncell + c] = fs * P.inv_dx;
+    double t = sdx * fs[v];
+    if (use_k) t = fma(rk1, uk[v], t);
+    if (use_n) t = fma(rk0, un[v], t);
     // a zero-length step (a run past its end time) leaves the state as it is
-    if (keep) {
-      Uo[v] = Uk[(long long)v * P.ncell + c];
-    } else {
-      double t = sdx * fs;
-      if (use_k) t = fma(rk1, Uk[(long long)v * P.ncell + c], t);
-      if (use_n) t = fma(rk0, Un[(long long)v * P.ncell + c], t);
-      Uo[v] = t;
-    }
+    Uo[v] = keep ? uk[v] : t;
   }
   if (Uout) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) Uout[(long long)v * P.ncell + c] = Uo[v];
-    if (!admissible<NS, D>(P, Uo)) atomicMax(status, (int)ST_INADMISSIBLE);
+    if (!admissible_cell<NS, D>(P, Uo)) atomicMax(status, (int)ST_INADMISSIBLE);
   }
 }
 
