@@ -27,7 +27,7 @@ namespace mpmc {
 
 // species constants as float-floats
 struct SpeciesFF {
-  ff R, cv, cp, pinf;
+  ff R, cv, cp, pinf, q, b;
 };
 
 MPMC_FF ff ff_of(double x) { return ff_scaled(x, 1023); }

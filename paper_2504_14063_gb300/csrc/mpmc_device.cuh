@@ -346,19 +346,14 @@ __device__ __forceinline__ void decode(const double* U, double& rho, double* Y, 
 // liquid, P to ~eps32 Pinf), from which one or two FP64 steps reach the
 // FP64 root.
 template <int NS>
-__device__ __forceinline__ double pt_start_f32(const KParams& P, const double* Y, const double* w, double Cv,
-                                               double lo, double x0) {
-  float wf[NS];
-#pragma unroll
-  for (int k = 0; k < NS; ++k) wf[k] = nonzero(Y[k]) ? narrow(w[k]) : 0.f;
-  const float cvf = narrow(Cv), lof = narrow(lo);
-  float x = narrow(x0), a = lof, b = INFINITY;
+__device__ __forceinline__ float pt_root_f32(const KParams& P, const float* wf, float cvf, float lof, float x) {
+  float a = lof, b = INFINITY;
   for (int it = 0; it < 40; ++it) {
     float f = -cvf, df = 0.f, d2f = 0.f, mag = cvf, rg = 0.f;
     bool have_rg = false;
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
-      if (nonzero(Y[k])) {
+      if (wf[k] != 0.f) {
         float r;
         if (P.f32.pinf[k] == 0.f) {
           if (!have_rg) {
@@ -386,7 +381,16 @@ __device__ __forceinline__ double pt_start_f32(const KParams& P, const double* Y
     x = xn;
     if (done || !(b > a)) break;
   }
-  return (double)x;
+  return x;
+}
+
+template <int NS>
+__device__ __forceinline__ double pt_start_f32(const KParams& P, const double* Y, const double* w, double Cv,
+                                               double lo, double x0) {
+  float wf[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) wf[k] = nonzero(Y[k]) ? narrow(w[k]) : 0.f;
+  return (double)pt_root_f32<NS>(P, wf, narrow(Cv), narrow(lo), narrow(x0));
 }
 
 // p-T equilibrium from mass fractions, specific internal energy and volume

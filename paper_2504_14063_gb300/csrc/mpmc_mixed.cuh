@@ -408,7 +408,193 @@ __device__ __forceinline__ void block_max2f(float a, float b, unsigned long long
   }
 }
 
-// per cell: FP64 inversion, FP32 cache
+// the primitive state of a cell, FP32
+template <int NS>
+struct CellF {
+  float rho, Y[NS], u[3], p, T;
+  int st;
+};
+
+// an FP64 value that ff_of splits exactly as narrow rounds it: in 2^-126 ..
+// 2^125 or zero, and not half way between two FP32 numbers (ff_of takes ties
+// away from zero)
+__device__ __forceinline__ bool in_f32(double x) {
+  const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu, l = (unsigned)__double2loint(x);
+  return (m - (897u << 20) < (251u << 20) && (l & 0x1fffffffu) != 0x10000000u) || (m | l) == 0u;
+}
+
+// a rounded to FP32; unsure: the bits below it come within `err` (relative to
+// half an ulp) of a tie, so that a's own error could turn the rounding
+__device__ __forceinline__ float ff_round(ff a, float err, bool& unsure) {
+  const float s = fadd(a.h, a.l), r = fadd(a.l, -fadd(s, -a.h));
+  const float hu = __uint_as_float(__float_as_uint(s) & 0x7f800000u) * 5.9604645e-8f;
+  unsure = unsure || fabsf(r) > hu * (1.f - err);
+  return s;
+}
+
+// decode and p-T equilibrium in FP64, for cells beyond the range of the
+// float-float form; out of line, so that it costs the pass no registers
+template <int NS, int D>
+__device__ __noinline__ void cell_fp64(const KParams& P, const double* __restrict__ U, long long stride,
+                                       CellF<NS>& o) {
+  constexpr int NV = NS + D + 1;
+  double Uc[NV], rho, Y[NS], u[3], e, vol, pd, Td;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) Uc[v] = U[(long long)v * stride];
+  decode<NS, D, false>(Uc, rho, Y, u, e, vol);
+  o.st = positive(rho) ? ST_OK : ST_INADMISSIBLE;
+#pragma unroll
+  for (int k = 0; k < NS; ++k)
+    if (Uc[k] < -YTOL * rho) o.st = ST_INADMISSIBLE;
+  const int st2 = pt_equilibrium<NS, false, true>(P, Y, e, vol, pd, Td, rho);
+  if (o.st == ST_OK) o.st = st2;
+  o.rho = narrow(rho);
+#pragma unroll
+  for (int k = 0; k < NS; ++k) o.Y[k] = narrow(Y[k]);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) o.u[d] = narrow(u[d]);
+  o.p = narrow(pd);
+  o.T = narrow(Td);
+}
+
+// The same in float-float on the FP32 pipe (about 2^-46 of every term, the
+// results then rounded to FP32).  The FP64 pipe bounded the pass: closed
+// forms with their divisions and root, or the several-liquid iteration.
+//   f(x) = sum_k w_k / (x + Pinf_k) - Cv,  w_k = Y_k R_k (E' - Pinf_k)
+// (NASG_T1 = NASG_T2) starts at the FP32 root of the quadratic with the
+// liquids merged into one, iterated in FP32 where they differ, and takes
+// Halley steps in float-float until one is below 1e-5 of the distance to the
+// nearest pole: what it leaves is of order 1e-15 of that distance.  The
+// rounding of a stiff liquid's terms leaves P within 2^-43 of the sum of their
+// magnitudes over the slope, a hundredth of P's FP32 rounding at P = 1e-4
+// Pinf; a result that comes that close to a rounding boundary is refused, so
+// that the FP32 cache holds what FP64 gives.  False (nothing written) there,
+// where the steps do not settle, and where a quantity leaves the range.
+template <int NS, int D>
+__device__ __forceinline__ bool cell_ff(const KParams& P, const ff* U, CellF<NS>& o) {
+  ff rho = U[0];
+#pragma unroll
+  for (int k = 1; k < NS; ++k) rho = ff_add(rho, U[k]);
+  if (!(rho.h > 1e-18f && rho.h < 1e18f)) return false;
+  const ff v = ff_rcp(rho);
+  ff ke = {0.f, 0.f}, u[D], Y[NS];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    u[d] = ff_mul(U[NS + d], v);
+    ke = ff_addp(ke, ff_sqr(u[d]));
+  }
+  ff em = ff_sub(ff_mul(U[NS + D], v), ff_mulf(ke, 0.5f)), vm = v, Cv = {0.f, 0.f};
+  float pmin = 3e38f, pl = -1.f, Rg = 0.f, Rl = 0.f, wpl = 0.f;
+  bool multi = false;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    Y[k] = ff_mul(U[k], v);
+    Cv = ff_add(Cv, ff_mul(Y[k], P.sff[k].cv));
+    if (P.has_q) em = ff_sub(em, ff_mul(Y[k], P.sff[k].q));
+    if (P.has_b) vm = ff_sub(vm, ff_mul(Y[k], P.sff[k].b));
+    if (Y[k].h > 0.f) {
+      const float pk = P.f32.pinf[k], yr = Y[k].h * P.f32.Rk[k];
+      pmin = fminf(pmin, pk);
+      if (pk > 0.f) {
+        if (pl < 0.f) pl = pk;
+        else if (pk != pl) multi = true;
+        Rl += yr;
+        wpl += yr * pk;
+      } else {
+        Rg += yr;
+      }
+    }
+  }
+  if (!(em.h > 0.f && vm.h > 0.f)) return false;
+  const ff Ep = P.has_b ? ff_mul(em, ff_rcp(vm)) : ff_mul(em, rho);
+  // (a species with Y <= 0 enters as in pt_equilibrium: with several liquids
+  // where Y is not zero, not otherwise)
+  ff w[NS];
+  float wf[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const bool on = multi ? Y[k].h != 0.f : Y[k].h > 0.f;
+    w[k] = on ? ff_mul(ff_mul(Y[k], P.sff[k].R), ff_sub(Ep, P.sff[k].pinf)) : ff{0.f, 0.f};
+    wf[k] = w[k].h;
+  }
+  const float lo = -pmin;
+  float x0;
+  {
+    const float pe = Rl > 0.f ? wpl * frcp(Rl) : 0.f;
+    const float a2 = Ep.h * (Rg + Rl) - pe * (Cv.h + Rl), a3 = Ep.h * pe * Rg;
+    const float sq = sqrtf(a2 * a2 + 4.f * Cv.h * a3);
+    x0 = a2 >= 0.f ? 0.5f * (a2 + sq) * frcp(Cv.h) : 2.f * a3 * frcp(sq - a2);
+  }
+  if (!(x0 > lo)) x0 = lo + fmaxf(fabsf(lo), 1.f);
+  if (multi) x0 = pt_root_f32<NS>(P, wf, Cv.h, lo, x0);
+  ff x = {x0, 0.f};
+  float err = 0.f;   // bound of x's rounding
+  bool done = false;
+  for (int it = 0; it < 4 && !done; ++it) {
+    ff f = {-Cv.h, -Cv.l};
+    float df = 0.f, d2 = 0.f, mag = Cv.h;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      if (wf[k] == 0.f) continue;
+      const ff r = ff_rcp(ff_add(x, P.sff[k].pinf)), t = ff_mul(w[k], r);
+      const float tr = t.h * r.h;
+      f = ff_add(f, t);
+      mag += fabsf(t.h);
+      df -= tr;
+      d2 += tr * r.h;
+    }
+    const float g = frcp(df), s = f.h * g, dx = -s * frcp(1.f - s * (d2 * g));
+    err = 1.1e-13f * mag * fabsf(g);
+    done = fabsf(dx) <= 1e-5f * (x.h - lo);
+    x = ff_add(x, ff{dx, 0.f});
+  }
+  if (!done || !(fabsf(x.h) < 1e18f && x.h > lo)) return false;
+  constexpr float E = 1.f / 65536.f;   // 2^-41 of a value
+  bool unsure = false;
+  const float p = ff_round(x, 0.f, unsure);
+  unsure = unsure || fabsf(x.l) + err > __uint_as_float(__float_as_uint(p) & 0x7f800000u) * 5.9604645e-8f;
+  float Yf[NS], T;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) Yf[k] = ff_round(Y[k], E, unsure);
+  if (multi) {
+    // in FP32, as pt_equilibrium's
+    float den = 0.f;
+#pragma unroll
+    for (int k = 0; k < NS; ++k)
+      if (Y[k].h != 0.f) {
+        const float r = P.f32.pinf[k] == 0.f
+                            ? 1.f
+                            : __fdividef(p + P.f32.gam[k] * P.f32.pinf[k], p + P.f32.pinf[k]);
+        den += Yf[k] * P.f32.cv[k] * r;
+      }
+    T = __fdividef(ff_round(em, E, unsure), den);
+  } else {
+    // T = (e - q) / (Cv + sum_k Y_k R_k Pinf_k / (P + Pinf_k))
+    ff den = Cv;
+#pragma unroll
+    for (int k = 0; k < NS; ++k)
+      if (Y[k].h != 0.f && P.f32.pinf[k] > 0.f)
+        den = ff_add(den, ff_mul(ff_mul(Y[k], P.sff[k].R), ff_mul(P.sff[k].pinf, ff_rcp(ff_add(x, P.sff[k].pinf)))));
+    T = ff_round(ff_mul(em, ff_rcp(den)), E, unsure);
+  }
+  if (!(fabsf(T) < 1e18f)) return false;
+  float uf[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) uf[d] = d < D ? ff_round(u[d], E, unsure) : 0.f;
+  const float rf = ff_round(rho, E, unsure);
+  if (unsure) return false;
+  o.p = p;
+  o.T = T;
+  o.rho = rf;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) o.Y[k] = Yf[k];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) o.u[d] = uf[d];
+  o.st = ST_OK;
+  return true;
+}
+
+// per cell: inversion of the FP64 state, FP32 cache
 template <int NS, int D>
 __global__ void __launch_bounds__(CELL_THREADS)
     k_prim(const KParams P, const double* __restrict__ U, const double* __restrict__ Uin, float* __restrict__ Wc,
@@ -417,51 +603,59 @@ __global__ void __launch_bounds__(CELL_THREADS)
   float smax = 0.f, gmax = 0.f;
   if (c < P.ncell + P.nextra) {
     constexpr int NV = NS + D + 1;
-    double Uc[NV];
-    if (c >= P.ncell) {
-      // the inflow state or a characteristic ghost, from U's ghost buffer
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Uc[v] = Uin[(long long)v * P.gstride + (c - P.ncell)];
-    } else {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Uc[v] = U[(long long)v * P.ncell + c];
-    }
+    // a cell, or the inflow state or a characteristic ghost from U's ghost buffer
+    const double* Up = c >= P.ncell ? Uin + (c - P.ncell) : U + c;
+    const long long us = c >= P.ncell ? P.gstride : P.ncell;
     const long long ws = P.wstride;
-    double rho, Y[NS], u[3], e, vol;
-    decode<NS, D, false>(Uc, rho, Y, u, e, vol);
-    int st = positive(rho) ? ST_OK : ST_INADMISSIBLE;
+    CellF<NS> q;
+    float Uf[NV];
+    {
+      ff Uc[NV];
+      bool range = true, neg = false;
 #pragma unroll
-    for (int k = 0; k < NS; ++k)
-      if (Uc[k] < -YTOL * rho) st = ST_INADMISSIBLE;
-    double pd, Td;
-    const int st2 = pt_equilibrium<NS, false, true>(P, Y, e, vol, pd, Td, rho);
-    if (st == ST_OK) st = st2;
+      for (int v = 0; v < NV; ++v) {
+        const double x = Up[(long long)v * us];
+        range = range && in_f32(x);
+        Uc[v] = ff_of(x);
+        Uf[v] = Uc[v].h;
+        neg = neg || (v < NS && Uc[v].h < 0.f);
+      }
+      if (!range || !cell_ff<NS, D>(P, Uc, q)) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Uf[v] = narrow(Up[(long long)v * us]);
+        cell_fp64<NS, D>(P, Up, us, q);
+      } else if (neg) {
+        double rho = Up[0];
+#pragma unroll
+        for (int k = 1; k < NS; ++k) rho += Up[(long long)k * us];
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+          if (Up[(long long)k * us] < -YTOL * rho) q.st = ST_INADMISSIBLE;
+      }
+    }
     SpeciesF sp[NS];
     load_species<NS>(P, sp);
-    float Yf[NS];
-#pragma unroll
-    for (int k = 0; k < NS; ++k) Yf[k] = narrow(Y[k]);
-    const float p = narrow(pd), T = narrow(Td);
+    const float* Yf = q.Y;
+    const float p = q.p, T = q.T;
     float r2, e2, a;
     eos_forward_f<NS>(sp, Yf, p, T, r2, e2, a);
     Wc[P.wT * ws + c] = T;
     Wc[P.wP * ws + c] = p;
-    Wc[P.wRho * ws + c] = narrow(rho);
+    Wc[P.wRho * ws + c] = q.rho;
     Wc[P.wA * ws + c] = a;
 #pragma unroll
     for (int k = 0; k < NS; ++k) Wc[(P.wY + k) * ws + c] = Yf[k];
 #pragma unroll
-    for (int d = 0; d < D; ++d) Wc[(P.wU + d) * ws + c] = narrow(u[d]);
+    for (int d = 0; d < D; ++d) Wc[(P.wU + d) * ws + c] = q.u[d];
     // FP32 copies of U for the limiter's first (FP32) admissibility test;
     // the pass that computes dt and Gamma (red != null) runs on U^n
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const float uf = narrow(Uc[v]);
-      Wc[(P.nW + v) * ws + c] = uf;
-      if (red) P.unf[v * ws + c] = uf;
+      Wc[(P.nW + v) * ws + c] = Uf[v];
+      if (red) P.unf[v * ws + c] = Uf[v];
     }
     float mu = 0.f, lam = 0.f;
-    const float rhof = narrow(rho);
+    const float rhof = q.rho;
     if (P.cdi || P.diffusion || P.viscous) {
       float phi[2], Yp[2];
 #pragma unroll
@@ -471,7 +665,7 @@ __global__ void __launch_bounds__(CELL_THREADS)
         for (int k = 0; k < NS; ++k)
           if (P.phase[k] == ph) {
             yp += Yf[k];
-            const float ry = narrow(Uc[k]);
+            const float ry = Uf[k];
             if (ry != 0.f) {
               f += ry * (sp[k].Rk * T / (p + sp[k].pinf) + sp[k].b);
               hr += ry * (sp[k].cp * T + sp[k].b * p + sp[k].q);
@@ -485,7 +679,7 @@ __global__ void __launch_bounds__(CELL_THREADS)
           Wc[(P.wHrho + ph) * ws + c] = present ? hr / f : 0.f;
 #pragma unroll
           for (int k = 0; k < NS; ++k)
-            if (P.phase[k] == ph) Wc[(P.wYrho + k) * ws + c] = present ? (float)Uc[k] / f : 0.f;
+            if (P.phase[k] == ph) Wc[(P.wYrho + k) * ws + c] = present ? Uf[k] / f : 0.f;
         }
       }
       if (P.cdi) {
@@ -541,12 +735,12 @@ __global__ void __launch_bounds__(CELL_THREADS)
         }
       }
     }
-    if (st != ST_OK) atomicMax(status, st);
+    if (q.st != ST_OK) atomicMax(status, q.st);
     if (c < P.ncell) {
       const float idx = P.f32.inv_dx;
 #pragma unroll
       for (int d = 0; d < D; ++d) {
-        const float ud = fabsf(narrow(u[d]));
+        const float ud = fabsf(q.u[d]);
         smax = fmaxf(smax, (ud + a) * idx);
         gmax = fmaxf(gmax, ud);
       }

@@ -89,6 +89,8 @@ inline int build_params(const mpmc_grid* g, const mpmc_eos* eos, const mpmc_mode
     P.sff[k].cv = split(P.cv[k]);
     P.sff[k].cp = split(P.cp[k]);
     P.sff[k].pinf = split(P.pinf[k]);
+    P.sff[k].q = split(P.q[k]);
+    P.sff[k].b = split(P.b[k]);
     if (eos->b[k] != 0.0) P.has_b = 1;
     if (eos->q[k] != 0.0) P.has_q = 1;
   }
