@@ -191,6 +191,12 @@ __device__ __forceinline__ CRef map_cell_dt(const KParams& P, int t, int i, int 
 
 __device__ __forceinline__ double sgn_flip(unsigned flip, int d) { return (flip >> d) & 1u ? -1.0 : 1.0; }
 
+// x, negated where bit d of flip is set, by its sign bit (a multiplication by
+// -1 issues on the FP64 pipe)
+__device__ __forceinline__ double mirror(double x, unsigned flip, int d) {
+  return __hiloint2double(__double2hiint(x) ^ (int)(((flip >> d) & 1u) << 31), __double2loint(x));
+}
+
 // conserved vector of a mapped cell (U has ncell entries per component; the
 // inflow state and the characteristic ghosts come from U's ghost buffer G)
 template <int NS, int D>
@@ -206,7 +212,7 @@ __device__ __forceinline__ void load_U(const KParams& P, const double* __restric
     for (int v = 0; v < NV; ++v) out[v] = U[(long long)v * P.ncell + r.idx];
   }
 #pragma unroll
-  for (int d = 0; d < D; ++d) out[NS + d] *= sgn_flip(r.flip, d);
+  for (int d = 0; d < D; ++d) out[NS + d] = mirror(out[NS + d], r.flip, d);
 }
 
 __device__ __forceinline__ double wget(const KParams& P, const double* __restrict__ Wc, int f, CRef r) {

@@ -541,66 +541,10 @@ __device__ __forceinline__ bool present_(double y) {
   return b >= __double_as_longlong(ABSENT) && b <= 0x7ff0000000000000ll;
 }
 
-// B (value) and M (sum of its terms' magnitudes) of one cell in FP32
-template <int NS, int D>
-__device__ __forceinline__ void limiter_base(const KParams& P, const double* __restrict__ Un,
-                                             const double* __restrict__ Uk, const double* __restrict__ Gk,
-                                             const CRef r, const float rk0, const float rk1, float* B, float* M) {
-  constexpr int NV = NS + D + 1;
-  const bool ghost = r.idx >= P.ncell;
-  const double* un = ghost ? P.gn + (r.idx - P.ncell) : Un + r.idx;
-  const double* uk = ghost ? Gk + (r.idx - P.ncell) : Uk + r.idx;
-  const long long st = ghost ? P.gstride : P.ncell;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    float a = rk0 * lim_narrow(un[(long long)v * st]);
-    float b = rk1 != 0.f ? rk1 * lim_narrow(uk[(long long)v * st]) : 0.f;
-    if (v >= NS && v < NS + D && ((r.flip >> (v - NS)) & 1u)) {
-      a = -a;
-      b = -b;
-    }
-    B[v] = a + b;
-    M[v] = fabsf(a) + fabsf(b);
-  }
-}
-
-template <int NS, int D>
-__device__ __noinline__ int admissible_fp32(const KParams& P, const float* B, const float* M, const float* F,
-                                               const float s) {
-  constexpr int NV = NS + D + 1;
-  float T[NV], G[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const float f = s * F[v];
-    T[v] = B[v] + f;
-    G[v] = M[v] + fabsf(f);
-  }
-  const int a = admissible_margin<NS, D>(P, T, G);
-  return fabsf(s) > LIM_TINY ? a : -1;
-}
-
-// the FP64 test of T = rk0 U^n + rk1 U^(k) + s F, for a flux that the FP32
-// one could not decide: out of line and from memory, so that it costs the
-// face kernel no registers
-template <int NS, int D>
-__device__ __noinline__ bool admissible_fp64(const KParams& P, const double* Un, const double* Uk, const double* Gk,
-                                             const CRef r, const double* F, const double rk0, const double rk1,
-                                             const double s) {
-  constexpr int NV = NS + D + 1;
-  double T[NV], B[NV];
-  load_U<NS, D>(P, Un, P.gn, r, B);
-  load_U<NS, D>(P, Uk, Gk, r, T);
-#pragma unroll
-  for (int v = 0; v < NV; ++v) T[v] = rk0 * B[v] + rk1 * T[v] + s * F[v];
-  return admissible<NS, D>(P, T);
-}
-
 // ---------------------------------------------------------------------------
-// velocity component t of a mapped cell, negated by its sign bit where a wall
-// mirrors it (a multiplication by -1 issues on the FP64 pipe)
+// velocity component t of a mapped cell, negated where a wall mirrors it
 __device__ __forceinline__ double uget(const KParams& P, const double* __restrict__ Wc, int t, CRef r) {
-  const double u = wget(P, Wc, P.wU + t, r);
-  return __hiloint2double(__double2hiint(u) ^ (int)(((r.flip >> t) & 1u) << 31), __double2loint(u));
+  return mirror(wget(P, Wc, P.wU + t, r), r.flip, t);
 }
 
 // ---------------------------------------------------------------------------
