@@ -1398,14 +1398,15 @@ struct AdjFaceImpl {
                    double* C) {
     long long nf = 1;
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
-    const unsigned nb = nblocks(nf, VJP_THREADS);
+    const int nt = block_threads(nf, VJP_THREADS);
+    const unsigned nb = nblocks(nf, nt);
     if (d == 0)
-      k_face_adj<NS, D, 0, RC><<<nb, VJP_THREADS, 0, s>>>(P, Wc, Uk, Uin, scal, tape, lamL, coef, mul_dt, C);
+      k_face_adj<NS, D, 0, RC><<<nb, nt, 0, s>>>(P, Wc, Uk, Uin, scal, tape, lamL, coef, mul_dt, C);
     else if (d == 1)
-      k_face_adj<NS, D, (D > 1 ? 1 : 0), RC><<<nb, VJP_THREADS, 0, s>>>(P, Wc, Uk, Uin, scal, tape, lamL, coef,
+      k_face_adj<NS, D, (D > 1 ? 1 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Uk, Uin, scal, tape, lamL, coef,
                                                                         mul_dt, C);
     else
-      k_face_adj<NS, D, (D > 2 ? 2 : 0), RC><<<nb, VJP_THREADS, 0, s>>>(P, Wc, Uk, Uin, scal, tape, lamL, coef,
+      k_face_adj<NS, D, (D > 2 ? 2 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Uk, Uin, scal, tape, lamL, coef,
                                                                         mul_dt, C);
   }
 };
@@ -1442,27 +1443,30 @@ struct AdjImpl {
                         const uint32_t* tape, const double* lamL, double coef, int mul_dt, double* C) {
     long long nf = 1;
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
-    const unsigned nb = nblocks(nf, VJP_THREADS);
+    const int nt = block_threads(nf, VJP_THREADS);
+    const unsigned nb = nblocks(nf, nt);
     if (d == 0)
-      k_face_visc_adj<NS, D, 0><<<nb, VJP_THREADS, 0, s>>>(P, Wc, scal, tape, lamL, coef, mul_dt, C);
+      k_face_visc_adj<NS, D, 0><<<nb, nt, 0, s>>>(P, Wc, scal, tape, lamL, coef, mul_dt, C);
     else if (d == 1)
-      k_face_visc_adj<NS, D, (D > 1 ? 1 : 0)><<<nb, VJP_THREADS, 0, s>>>(P, Wc, scal, tape, lamL, coef, mul_dt, C);
+      k_face_visc_adj<NS, D, (D > 1 ? 1 : 0)><<<nb, nt, 0, s>>>(P, Wc, scal, tape, lamL, coef, mul_dt, C);
     else
-      k_face_visc_adj<NS, D, (D > 2 ? 2 : 0)><<<nb, VJP_THREADS, 0, s>>>(P, Wc, scal, tape, lamL, coef, mul_dt, C);
+      k_face_visc_adj<NS, D, (D > 2 ? 2 : 0)><<<nb, nt, 0, s>>>(P, Wc, scal, tape, lamL, coef, mul_dt, C);
   }
   static void gather(const KParams& P, cudaStream_t s, int d, const double* C, int first, double* gW, double* gU) {
-    const unsigned nb = nblocks(P.ncell, CELL_THREADS);
+    const int nt = block_threads(P.ncell, CELL_THREADS);
+    const unsigned nb = nblocks(P.ncell, nt);
     if (d == 0)
-      k_gather<NS, D, 0><<<nb, CELL_THREADS, 0, s>>>(P, C, first, gW, gU);
+      k_gather<NS, D, 0><<<nb, nt, 0, s>>>(P, C, first, gW, gU);
     else if (d == 1)
-      k_gather<NS, D, (D > 1 ? 1 : 0)><<<nb, CELL_THREADS, 0, s>>>(P, C, first, gW, gU);
+      k_gather<NS, D, (D > 1 ? 1 : 0)><<<nb, nt, 0, s>>>(P, C, first, gW, gU);
     else
-      k_gather<NS, D, (D > 2 ? 2 : 0)><<<nb, CELL_THREADS, 0, s>>>(P, C, first, gW, gU);
+      k_gather<NS, D, (D > 2 ? 2 : 0)><<<nb, nt, 0, s>>>(P, C, first, gW, gU);
   }
   static void cell(const KParams& P, cudaStream_t s, const double* U, const double* Wc, const double* gW,
                    const double* gU, double* out, double a, const double* x, double b, const double* y, double cz,
                    const double* z) {
-    k_cell_adj<NS, D><<<nblocks(P.ncell, CELL_THREADS), CELL_THREADS, 0, s>>>(P, U, Wc, gW, gU, out, a, x, b, y,
+    const int nt = block_threads(P.ncell, CELL_THREADS);
+    k_cell_adj<NS, D><<<nblocks(P.ncell, nt), nt, 0, s>>>(P, U, Wc, gW, gU, out, a, x, b, y,
                                                                                cz, z);
   }
   static void init(const KParams& P, cudaStream_t s, const double* prim, const double* lamU, double* lprim,

@@ -993,7 +993,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
 template <int NS, int D>
 void prim(const KParams& P, cudaStream_t s, const double* U, const double* Uin, double* Wc, unsigned long long* red,
           int* status) {
-  fast::k_prim<NS, D><<<nblocks(P.ncell + P.nextra, CELL_THREADS), CELL_THREADS, 0, s>>>(P, U, Uin, Wc, red, status);
+  const int nt = block_threads(P.ncell + P.nextra, CELL_THREADS);
+  fast::k_prim<NS, D><<<nblocks(P.ncell + P.nextra, nt), nt, 0, s>>>(P, U, Uin, Wc, red, status);
 }
 
 // the forward FP64 face pass of one direction with interpolation RC
@@ -1004,14 +1005,15 @@ struct FaceImpl {
                    uint32_t* flags, unsigned long long* stats) {
     long long nf = 1;
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
-    const unsigned nb = nblocks(nf, FACE_THREADS);
+    const int nt = block_threads(nf, FACE_THREADS);
+    const unsigned nb = nblocks(nf, nt);
     if (d == 0)
-      fast::k_face<NS, D, 0, RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F, flags, stats);
+      fast::k_face<NS, D, 0, RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F, flags, stats);
     else if (d == 1)
-      fast::k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+      fast::k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
                                                                      flags, stats);
     else
-      fast::k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+      fast::k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
                                                                      flags, stats);
   }
 };

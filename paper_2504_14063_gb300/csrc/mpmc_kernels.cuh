@@ -750,8 +750,6 @@ __global__ void __launch_bounds__(CELL_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------
-inline unsigned nblocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
-
 // the FP64 face pass of one direction with interpolation RC
 template <int NS, int D, int RC>
 struct FaceImpl {
@@ -760,14 +758,15 @@ struct FaceImpl {
                    uint32_t* flags, unsigned long long* stats) {
     long long nf = 1;
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
-    const unsigned nb = nblocks(nf, FACE_THREADS);
+    const int nt = block_threads(nf, FACE_THREADS);
+    const unsigned nb = nblocks(nf, nt);
     if (d == 0)
-      k_face<NS, D, 0, RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F, flags, stats);
+      k_face<NS, D, 0, RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F, flags, stats);
     else if (d == 1)
-      k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+      k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
                                                                      flags, stats);
     else
-      k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+      k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
                                                                      flags, stats);
   }
 };
@@ -799,7 +798,8 @@ struct Impl {
   }
   static void prim(const KParams& P, cudaStream_t s, const double* U, const double* Uin, double* Wc,
                    unsigned long long* red, int* status) {
-    k_prim<NS, D><<<nblocks(P.ncell + P.nextra, CELL_THREADS), CELL_THREADS, 0, s>>>(P, U, Uin, Wc, red,
+    const int nt = block_threads(P.ncell + P.nextra, CELL_THREADS);
+    k_prim<NS, D><<<nblocks(P.ncell + P.nextra, nt), nt, 0, s>>>(P, U, Uin, Wc, red,
                                                                                             status);
   }
   static void face(const KParams& P, cudaStream_t s, int d, const double* Wc, const double* Un, const double* Uk,
@@ -810,7 +810,8 @@ struct Impl {
   static void update(const KParams& P, cudaStream_t s, const double* Un, const double* Uk, double* const* F,
                      const double* scal, double rk0, double rk1, double rk2, double* Uout, double* dUdt,
                      int* status) {
-    k_update<NS, D><<<nblocks(P.ncell, CELL_THREADS), CELL_THREADS, 0, s>>>(
+    const int nt = block_threads(P.ncell, CELL_THREADS);
+    k_update<NS, D><<<nblocks(P.ncell, nt), nt, 0, s>>>(
         P, Un, Uk, F[0], D > 1 ? F[1] : F[0], D > 2 ? F[2] : F[0], scal, rk0, rk1, rk2, Uout, dUdt, status);
   }
   static void ghost(const KParams& P, cudaStream_t s, const double* U, double* G) {

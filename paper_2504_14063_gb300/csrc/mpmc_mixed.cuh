@@ -1274,8 +1274,6 @@ __global__ void __launch_bounds__(CELL_THREADS, 3)
   update_cell<NS, D>(P, c, Un, Uk, F0, F1, F2, scal, rk0, rk1, rk2, Uout, dUdt, status);
 }
 
-inline unsigned nblocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
-
 // the mixed face pass of one direction with interpolation RC
 template <int NS, int D, int RC>
 struct FaceImpl {
@@ -1284,16 +1282,17 @@ struct FaceImpl {
                    uint32_t* flags, unsigned long long* stats) {
     long long nf = 1;
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
-    const unsigned nb = nblocks(nf, FACE_THREADS);
+    const int nt = block_threads(nf, FACE_THREADS);
+    const unsigned nb = nblocks(nf, nt);
     const float* W = reinterpret_cast<const float*>(Wc);
     float* Ff = reinterpret_cast<float*>(F);   // the mixed path's fluxes are FP32
     if (d == 0)
-      k_face<NS, D, 0, RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff, flags, stats);
+      k_face<NS, D, 0, RC><<<nb, nt, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff, flags, stats);
     else if (d == 1)
-      k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff,
+      k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, nt, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff,
                                                                      flags, stats);
     else
-      k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, FACE_THREADS, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff,
+      k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, nt, 0, s>>>(P, W, Un, Uk, Uin, scal, rk0, rk1, rk2, Ff,
                                                                      flags, stats);
   }
 };
@@ -1322,8 +1321,8 @@ template <int NS, int D>
 struct Impl {
   static void prim(const KParams& P, cudaStream_t s, const double* U, const double* Uin, double* Wc,
                    unsigned long long* red, int* status) {
-    k_prim<NS, D><<<nblocks(P.ncell + P.nextra, CELL_THREADS), CELL_THREADS, 0, s>>>(
-        P, U, Uin, reinterpret_cast<float*>(Wc), red, status);
+    const int nt = block_threads(P.ncell + P.nextra, CELL_THREADS);
+    k_prim<NS, D><<<nblocks(P.ncell + P.nextra, nt), nt, 0, s>>>(P, U, Uin, reinterpret_cast<float*>(Wc), red, status);
   }
   static void face(const KParams& P, cudaStream_t s, int d, const double* Wc, const double* Un, const double* Uk,
                    const double* Uin, const double* scal, double rk0, double rk1, double rk2, double* F,
@@ -1335,7 +1334,8 @@ struct Impl {
                      int* status) {
     const float* Ff[3];
     for (int d = 0; d < 3; ++d) Ff[d] = reinterpret_cast<const float*>(F[d < D ? d : 0]);
-    k_update<NS, D><<<nblocks(P.ncell, CELL_THREADS), CELL_THREADS, 0, s>>>(P, Un, Uk, Ff[0], Ff[1], Ff[2], scal,
+    const int nt = block_threads(P.ncell, CELL_THREADS);
+    k_update<NS, D><<<nblocks(P.ncell, nt), nt, 0, s>>>(P, Un, Uk, Ff[0], Ff[1], Ff[2], scal,
                                                                             rk0, rk1, rk2, Uout, dUdt, status);
   }
 };

@@ -8,6 +8,16 @@ namespace mpmc {
 
 struct KParams;
 
+// Threads per block of a pass over n cells or faces that takes `most` on large
+// grids.  Blocks of one warp spread a small grid over more SMs, each with an
+// FP64 pipe of its own, and leave a smaller last wave: slab of 400 cells, 20
+// steps 2.24 -> 2.03 ms, reverse step of a 201 x 103 box 3.30 -> 2.38 ms,
+// 301 x 203 right-hand side 240 -> 219 us.  Beyond eight full blocks per SM the
+// waves are many and full blocks share more of their stencils in L1: 512 x 512
+// adjoint faces 9.1 ms (9.9 with one warp), 256^3 mixed faces 36.7 (38.5).
+inline int block_threads(long long n, int most) { return n < 152ll * 8 * most ? 32 : most; }
+inline unsigned nblocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
+
 struct Ops {
   void (*init)(const KParams&, cudaStream_t, const double* prim, double* U, long long n);
   void (*prim)(const KParams&, cudaStream_t, const double* U, const double* Uin, double* Wc,
