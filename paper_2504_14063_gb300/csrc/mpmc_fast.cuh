@@ -590,8 +590,17 @@ __device__ __noinline__ double2 face_avg_fp64(const KParams& P, const double* Wc
 // Four blocks per SM (128 registers): more warps hide the latencies of the
 // FP64 and FP32 chains (three or two blocks, unbounded registers: 20 % slower;
 // five and six, with spills: within 5 % either way).
-template <int NS, int D, int DIR, int RC>
-__global__ void __launch_bounds__(FACE_THREADS, 4)
+// SPLIT: a block is 32 faces x one warp per interpolated field (in the order
+// T, u_d + and -, Y_k, u_t): every warp forms X and c and interpolates its
+// field, the second builds the right states beside the first's left ones, the
+// first finishes the faces.  On a grid that leaves most warp slots empty the
+// pass lasts as long as one thread's chain of operations, which this shortens:
+// 100 and 400 cells in 1D, per pass 31 -> 24 and 27 -> 20 us (the same bits).
+template <int NS, int D>
+constexpr int SPLIT_WARPS = 3 + NS + (D - 1);
+
+template <int NS, int D, int DIR, int RC, bool SPLIT = false>
+__global__ void __launch_bounds__(SPLIT ? 32 * SPLIT_WARPS<NS, D> : FACE_THREADS, SPLIT ? 1 : 4)
     k_face(const __grid_constant__ KParams P, const double* __restrict__ Wc, const double* __restrict__ Un,
            const double* __restrict__ Uk, const double* __restrict__ Uin, const double* __restrict__ scal,
            const double rk0, const double rk1, const double rk2, double* __restrict__ F,
@@ -600,8 +609,12 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   constexpr int d = DIR;
   const int f0 = P.n[0] + (d == 0), f1 = P.n[1] + (d == 1), f2 = P.n[2] + (d == 2);
   const long long nf = (long long)f0 * f1 * f2;
-  const long long fid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (fid >= nf) return;
+  const int role = SPLIT ? (int)threadIdx.x >> 5 : 0, lane = (int)threadIdx.x & 31;
+  // (split: lanes beyond the last face repeat it, unstored)
+  long long fid = SPLIT ? (long long)blockIdx.x * 32 + lane : (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool live = fid < nf;
+  if (SPLIT) fid = live ? fid : nf - 1;
+  else if (!live) return;
   int fc[3];
   unflatten(fid, f0, f1, fc);
   int ci[3] = {fc[0], fc[1], fc[2]};
@@ -645,6 +658,50 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   // steps 2-3: project, interpolate both sides (WENO5-Z unless RC says
   // otherwise), back to physical space
   double YL[NS], YR[NS], uL[3] = {0.0, 0.0, 0.0}, uR[3] = {0.0, 0.0, 0.0}, PL, PR, TL, TR;
+  if constexpr (SPLIT) {
+    constexpr int NFLD = SPLIT_WARPS<NS, D>;
+    __shared__ double sh[2][NFLD][32];
+    {
+      double y[6];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) {
+        if (role < 3) {
+          const double p = wget(P, Wc, P.wP, cr[j]);
+          if (role == 0) y[j] = fma(-X, p, wget(P, Wc, P.wT, cr[j]));
+          else y[j] = fma(role == 1 ? c : -c, uget(P, Wc, d, cr[j]), p);
+        } else if (role < 3 + NS) {
+          y[j] = wget(P, Wc, P.wY + role - 3, cr[j]);
+        } else {
+          // the tangential directions in increasing order
+          const int q = role - 3 - NS, t = q < d ? q : q + 1;
+          y[j] = uget(P, Wc, t, cr[j]);
+        }
+      }
+      const double2 v = eno_lr<RC>(y[0], y[1], y[2], y[3], y[4], y[5], P.weno_eps4.h, P.weno_eps4.l, P.weno_eps4.e,
+                                   role == 1 || role == 2 ? 1 : 0);
+      sh[0][role][lane] = v.x;
+      sh[1][role][lane] = v.y;
+    }
+    __syncthreads();
+    PL = 0.5 * (sh[0][1][lane] + sh[0][2][lane]);
+    PR = 0.5 * (sh[1][1][lane] + sh[1][2][lane]);
+    TL = fma(X, PL, sh[0][0][lane]);
+    TR = fma(X, PR, sh[1][0][lane]);
+    uL[d] = (0.5 * ic) * (sh[0][1][lane] - sh[0][2][lane]);
+    uR[d] = (0.5 * ic) * (sh[1][1][lane] - sh[1][2][lane]);
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      YL[k] = sh[0][3 + k][lane];
+      YR[k] = sh[1][3 + k][lane];
+    }
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+      if (t == d) continue;
+      const int q = 3 + NS + (t < d ? t : t - 1);
+      uL[t] = sh[0][q][lane];
+      uR[t] = sh[1][q][lane];
+    }
+  } else {
   {
     double w1[6], w5[6], w6[6];
 #pragma unroll
@@ -684,6 +741,8 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
     fast::recon_lr<RC>(P, y, uL[t], uR[t]);
   }
 
+  }
+
   // cell values of the two face neighbours
   double Yi[NS], Yj[NS];
 #pragma unroll
@@ -714,8 +773,22 @@ __global__ void __launch_bounds__(FACE_THREADS, 4)
   double Fx[NV];
   {
     State<NS> sL, sR;
-    face_state<NS>(P, YL, uL, PL, TL, sL);
-    face_state<NS>(P, YR, uR, PR, TR, sR);
+    if constexpr (SPLIT) {
+      // the second warp builds the right state; the others are done
+      __shared__ State<NS> sh[32];
+      if (role == 1) {
+        face_state<NS>(P, YR, uR, PR, TR, sR);
+        sh[lane] = sR;
+      } else if (role == 0) {
+        face_state<NS>(P, YL, uL, PL, TL, sL);
+      }
+      __syncthreads();
+      if (role != 0 || !live) return;
+      sR = sh[lane];
+    } else {
+      face_state<NS>(P, YL, uL, PL, TL, sL);
+      face_state<NS>(P, YR, uR, PR, TR, sR);
+    }
     hllc_flux<NS, D>(d, sL, sR, Fx);
   }
 
@@ -1005,6 +1078,21 @@ struct FaceImpl {
                    uint32_t* flags, unsigned long long* stats) {
     long long nf = 1;
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
+    if constexpr (D < 3) {
+      // up to two split blocks per SM; with more the redundant X and c cost more
+      // than the shorter chain gives (TENO6 faces of 322 x 51 cells: 130 us whole,
+      // 274 us split; 5996 cells: 58 whole, 56 split)
+      if (nf <= 2 * 152 * 32) {
+        constexpr int nt = 32 * SPLIT_WARPS<NS, D>;
+        if (d == 0)
+          fast::k_face<NS, D, 0, RC, true><<<nblocks(nf, 32), nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
+                 flags, stats);
+        else
+          fast::k_face<NS, D, (D > 1 ? 1 : 0), RC, true><<<nblocks(nf, 32), nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal,
+                 rk0, rk1, rk2, F, flags, stats);
+        return;
+      }
+    }
     const int nt = block_threads(nf, FACE_THREADS);
     const unsigned nb = nblocks(nf, nt);
     if (d == 0)
