@@ -27,6 +27,7 @@ struct mpmc_ctx {
   cudaStream_t cap;  // internal stream used only to capture graphs
   int device;
   double* Wc = nullptr;
+  double* Wc2 = nullptr;  // a second cache, for the reverse step (first use)
   double* F[3] = {nullptr, nullptr, nullptr};
   long long nface[3] = {0, 0, 0};
   long long nface_total = 0;
@@ -156,7 +157,8 @@ static void free_all(mpmc_ctx* c) {
   // g_U and g_hist are caller-owned and never freed here
   void* ptrs[] = {c->Wc,   c->F[0],  c->F[1],    c->F[2],   c->U1,   c->U2,   c->Ud,   c->Uin,
                   c->scal, c->red,   c->status,  c->stats,  c->counter, c->gW, c->lamA, c->lamB,
-                  c->tape_int, c->Cslots, c->gU, c->unf, c->Gk != c->Uin ? c->Gk : nullptr};
+                  c->tape_int, c->Cslots, c->gU, c->unf, c->Wc2,
+                  c->Gk != c->Uin ? c->Gk : nullptr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
@@ -472,6 +474,10 @@ static int ensure_adjoint(mpmc_ctx* c) {
   long long nfmax = 0;
   for (int d = 0; d < P.dim; ++d) nfmax = c->nface[d] > nfmax ? c->nface[d] : nfmax;
   if (!c->Cslots) rc = alloc(c, (void**)&c->Cslots, (size_t)c->aops.slots(P) * nfmax * sizeof(double));
+  if (!rc && !c->Wc2 && cudaMalloc((void**)&c->Wc2, (size_t)P.nW * P.wstride * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    c->Wc2 = nullptr;   // the reverse step then recomputes U^n's cache
+  }
   if (!rc && !c->gW) rc = alloc(c, (void**)&c->gW, (size_t)P.nW * P.wstride * sizeof(double));
   if (!rc && !c->gU) rc = alloc(c, (void**)&c->gU, st_bytes);
   if (!rc && !c->lamA) rc = alloc(c, (void**)&c->lamA, st_bytes);
@@ -581,6 +587,17 @@ extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double
   const KParams& P = c->P;
   const long long nf = c->nface_total, n = (long long)P.nv * P.ncell;
   cudaStream_t s = c->stream;
+  // Gamma needs U^n's primitive pass first and the reverse of its stage comes
+  // last: its cache stays where it is and the stage states' go to a second one
+  // (a pass of its own for U^n at the end was one of four: recorded step and
+  // reverse at 512 x 512 16.13 -> 15.95 ms)
+  // (without memory for it, as before)
+  auto other_cache = [&] {
+    if (W_stages || !c->Wc2) return;
+    double* w = c->Wc;
+    c->Wc = c->Wc2;
+    c->Wc2 = w;
+  };
   dt_gamma(c, c->rec, s, U_n, dt, -1.0, nullptr);
   const double* U1 = U_stages ? U_stages : c->U1;
   const double* U2 = U_stages ? U_stages + n : c->U2;
@@ -588,6 +605,7 @@ extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double
   if (!U_stages) {
     // forward recomputation of the stage states (and of the flags if no tape)
     stage(c, c->rec, s, U_n, U_n, 1.0, 0.0, 1.0, c->U1, nullptr, tp);
+    other_cache();
     prim(c, c->rec, s, c->U1, nullptr);
     stage(c, c->rec, s, U_n, c->U1, 0.75, 0.25, 0.25, c->U2, nullptr, tp ? tp + nf : nullptr);
     prim(c, c->rec, s, c->U2, nullptr);
@@ -595,11 +613,13 @@ extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double
   } else if (tp) {
     // stage states given, flags recomputed
     faces_only(c, s, U_n, U_n, 1.0, 0.0, 1.0, tp);
+    other_cache();
     prim(c, c->rec, s, U1, nullptr);
     faces_only(c, s, U_n, U1, 0.75, 0.25, 0.25, tp + nf);
     prim(c, c->rec, s, U2, nullptr);
     faces_only(c, s, U_n, U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, tp + 2 * nf);
   } else if (!W_stages) {
+    other_cache();
     prim(c, c->rec, s, U2, nullptr);
   }
   const uint32_t* T = tape ? tape : c->tape_int;
@@ -618,8 +638,9 @@ extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double
   if (!W_stages) prim(c, c->rec, s, U1, nullptr);
   stage_vjp(c, s, U1, W_stages ? W_stages + nw : Wc, T + nf, l2, 0.25, 1, l1, 0.25, l2, 0.0, nullptr, 0.0,
             nullptr);
-  if (!W_stages) prim(c, c->rec, s, U_n, nullptr);
-  stage_vjp(c, s, U_n, W_stages ? W_stages : Wc, T, l1, 1.0, 1, lam_n, 1.0 / 3.0, lam_next, 0.75, l2, 1.0, l1);
+  other_cache();
+  if (!W_stages && !c->Wc2) prim(c, c->rec, s, U_n, nullptr);
+  stage_vjp(c, s, U_n, W_stages ? W_stages : c->Wc, T, l1, 1.0, 1, lam_n, 1.0 / 3.0, lam_next, 0.75, l2, 1.0, l1);
   return check_launch(c, "rk_step_adjoint");
 }
 
