@@ -80,8 +80,9 @@ extern "C" {
 
 /* precision of the hot path */
 #define MPMC_FP64 0
-#define MPMC_MIXED 1 /* reconstruction, fluxes, diffusion in FP32; EOS inversion,
-                        positivity bounds and RK accumulation in FP64 */
+#define MPMC_MIXED 1 /* reconstruction, fluxes, diffusion in FP32; EOS inversion to
+                        FP64's result rounded to FP32 (float-float, FP64 where that is
+                        in doubt); positivity bounds and RK accumulation in FP64 */
 
 /* per-face tape bits (mpmc_rk_step tape, mpmc_rhs flags) */
 #define MPMC_F_THETA_T_L (1u << 0) /* left T fell back to the cell value (Sec. 3.3.1) */
@@ -243,6 +244,10 @@ int mpmc_rhs_adjoint(mpmc_ctx* ctx, const double* U, const mpmc_stage* stage, co
  * contexts only, else MPMC_INVALID_ARG) the primitive caches of U^n, U^(1)
  * and U^(2), which spare the reverse step their recomputation. */
 int mpmc_rk_step_record(mpmc_ctx* ctx, double* U, double dt, uint32_t* tape, double* U_stages, double* W_stages);
+
+/* The same; dt_out (nullable, device double) receives the step's length. */
+int mpmc_rk_step_record_dt(mpmc_ctx* ctx, double* U, double dt, uint32_t* tape, double* U_stages, double* W_stages,
+                           double* dt_out);
 
 /* One SSP-RK3 step in place in the arithmetic of mpmc_rk_step_record (bit for
  * bit the states that it records; mpmc_rk_step and mpmc_step_n round

@@ -18,7 +18,9 @@ pass are replayed and each step's dt and Gamma are frozen (Sec. 3.3, 3.4).
         probe).  The backward pass replays each segment from its checkpoint
         (one forward step per step, keeping each step's input, stage states
         and limiter flags) and sweeps it in reverse, so memory holds the
-        checkpoints plus one segment of inputs, stage states and flags.
+        checkpoints plus one segment of inputs, stage states and flags.  The
+        last segment, which the backward pass takes first, is recorded by the
+        forward pass itself where it fits in an eighth of the free memory.
 """
 import torch
 
@@ -86,26 +88,58 @@ def _probe_term(ctx, U, probe):
     return (ctx.primitives(U)[1] * probe).sum()
 
 
+def _segment(ctx, m, like, share=None):
+    """(step inputs and last output, stage states, flags, primitive caches or
+    None) of m steps; None where the first three exceed `share` of the
+    device's free memory (share None: no limit, and caches by their own)."""
+    shape = tuple(like.shape)
+    if share is not None:
+        free, _ = torch.cuda.mem_get_info(like.device)
+        nbytes = (3 * m + 1) * like.numel() * 8 + m * 3 * ctx.nfaces_total * 4
+        caches = m * 3 * ctx.cache_doubles * 8
+        if nbytes > share * free:
+            return None
+        wst = _stage_caches(ctx, m, like.device, share) if nbytes + caches <= share * free else None
+    return (torch.empty((m + 1,) + shape, dtype=like.dtype, device=like.device),
+            torch.empty((m, 2) + shape, dtype=like.dtype, device=like.device),
+            torch.empty((m, 3 * ctx.nfaces_total), dtype=torch.int32, device=like.device),
+            wst if share is not None else _stage_caches(ctx, m, like.device))
+
+
 class _Rollout(torch.autograd.Function):
     @staticmethod
-    def forward(fctx, ctx, U0, n, every, probe, dt):
+    def forward(fctx, ctx, U0, n, every, probe, dt, grad):
         U = U0.detach().contiguous().clone()
         ckpts = []
         dts = torch.empty(n, dtype=torch.float64, device=U.device)
         slot = torch.empty(1, dtype=torch.float64, device=U.device)
         J = torch.zeros((), dtype=torch.float64, device=U.device)
+        # the last segment, kept for the backward pass (it would replay it
+        # first, bit for bit: half of the replayed steps of a rollout of two
+        # segments, 192 x 192, 20 steps)
+        last = (n - 1) // every * every
+        kept = _segment(ctx, n - last, U, 0.125) if grad and n > 0 else None
         for k in range(n):
             if k % every == 0:
                 ckpts.append(U.clone())
             # a step of fixed length, or the CFL step of U^k, recorded
-            ctx.rk_step_replay(U, dt, slot)
+            if kept is not None and k >= last:
+                q = k - last
+                states, stages, tapes, wst = kept
+                if q == 0:
+                    states[0].copy_(U)
+                states[q + 1].copy_(states[q])
+                U = states[q + 1]
+                ctx.rk_step_record(U, dt, tapes[q], stages[q], wst[q] if wst is not None else None, slot)
+            else:
+                ctx.rk_step_replay(U, dt, slot)
             dts[k] = slot[0]
             if probe is not None:
                 J += dts[k] * _probe_term(ctx, U, probe)
         fctx.ctx, fctx.n, fctx.every, fctx.probe = ctx, n, every, probe
-        fctx.ckpts, fctx.dts = ckpts, dts
+        fctx.ckpts, fctx.dts, fctx.kept = ckpts, dts, kept
         fctx.mark_non_differentiable(dts)
-        return U, J, dts
+        return U.clone() if kept is not None else U, J, dts
 
     @staticmethod
     def backward(fctx, gU, gJ, _gdts):
@@ -117,20 +151,20 @@ class _Rollout(torch.autograd.Function):
         if probe is not None and gJ != 0.0:
             lamW = torch.zeros((len(ctx.prim_fields),) + tuple(lam.shape[1:]), dtype=torch.float64,
                                device=lam.device)
-        nf = ctx.nfaces_total
         for seg in reversed(range(len(fctx.ckpts))):
             k0, k1 = seg * every, min(n, (seg + 1) * every)
             m = k1 - k0
-            # replay the segment, keeping every step's input, stage states and flags
-            states = torch.empty((m + 1,) + tuple(lam.shape), dtype=lam.dtype, device=lam.device)
-            stages = torch.empty((m, 2) + tuple(lam.shape), dtype=lam.dtype, device=lam.device)
-            tapes = torch.empty((m, 3 * nf), dtype=torch.int32, device=lam.device)
-            wst = _stage_caches(ctx, m, lam.device)
-            states[0].copy_(fctx.ckpts[seg])
-            for q in range(m):
-                states[q + 1].copy_(states[q])
-                ctx.rk_step_record(states[q + 1], dt_host[k0 + q], tapes[q], stages[q],
-                                   wst[q] if wst is not None else None)
+            if fctx.kept is not None and seg == len(fctx.ckpts) - 1:
+                states, stages, tapes, wst = fctx.kept
+                fctx.kept = None   # (another backward pass replays it)
+            else:
+                # replay the segment, keeping every step's input, stage states and flags
+                states, stages, tapes, wst = _segment(ctx, m, lam)
+                states[0].copy_(fctx.ckpts[seg])
+                for q in range(m):
+                    states[q + 1].copy_(states[q])
+                    ctx.rk_step_record(states[q + 1], dt_host[k0 + q], tapes[q], stages[q],
+                                       wst[q] if wst is not None else None)
             for q in reversed(range(m)):
                 k = k0 + q
                 if lamW is not None:
@@ -139,7 +173,7 @@ class _Rollout(torch.autograd.Function):
                     ctx.primitives_adjoint(states[q + 1], lamW, lam)
                 ctx.rk_step_adjoint(states[q], lam, dt=dt_host[k], tape=tapes[q], lam_n=lam, stages=stages[q],
                                     wstages=wst[q] if wst is not None else None)
-        return None, lam, None, None, None, None
+        return None, lam, None, None, None, None, None
 
 
 def init_state(ctx, prim):
@@ -159,7 +193,8 @@ def rollout(ctx, U0, n, every=20, probe=None, dt=0.0):
     step of its own U^k (recorded, and frozen in the backward pass)."""
     if ctx.precision != _b.FP64:
         raise ValueError("the discrete adjoint needs an FP64 context")
-    return _Rollout.apply(ctx, U0, int(n), int(every), probe, float(dt))
+    grad = torch.is_grad_enabled() and U0.requires_grad
+    return _Rollout.apply(ctx, U0, int(n), int(every), probe, float(dt), grad)
 
 
 # the autograd Function of one step, for callers that chain steps themselves

@@ -79,6 +79,7 @@ def _load():
         "mpmc_dt_gamma": (i, [vp, vp, vp]),
         "mpmc_rhs_adjoint": (i, [vp, vp, ctypes.POINTER(StageC), vp, vp, vp]),
         "mpmc_rk_step_record": (i, [vp, vp, d, vp, vp, vp]),
+        "mpmc_rk_step_record_dt": (i, [vp, vp, d, vp, vp, vp, vp]),
         "mpmc_rk_step_replay": (i, [vp, vp, d, vp]),
         "mpmc_rk_step_adjoint": (i, [vp, vp, vp, vp, d, vp, vp, vp]),
         "mpmc_init_state_adjoint": (i, [vp, vp, vp, vp]),
@@ -272,14 +273,14 @@ class Context:
             raise ValueError("wstages: a contiguous CUDA float64 tensor of at least 3 x cache_doubles elements")
         return w.data_ptr()
 
-    def rk_step_record(self, U, dt=0.0, tape=None, stages=None, wstages=None):
+    def rk_step_record(self, U, dt=0.0, tape=None, stages=None, wstages=None, dt_out=None):
         """One SSP-RK3 step in place that also returns its stage states
-        (2 x state: U^(1), U^(2)) and fills `tape` (3 x faces uint32) and
+        (2 x state: U^(1), U^(2)) and fills `tape` (3 x faces uint32),
         `wstages` (3 x cache_doubles FP64: the primitive caches of U^n, U^(1),
-        U^(2)) if given."""
+        U^(2)) and `dt_out` (1 double, device: the step's length) if given."""
         stages = torch.empty((2,) + tuple(U.shape), dtype=U.dtype, device=U.device) if stages is None else stages
-        self._check(lib.mpmc_rk_step_record(self.h, _dev(U), float(dt), _ptr(tape), _dev(stages),
-                                            self._wstages(wstages)))
+        self._check(lib.mpmc_rk_step_record_dt(self.h, _dev(U), float(dt), _ptr(tape), _dev(stages),
+                                               self._wstages(wstages), _ptr(dt_out)))
         return stages
 
     def rk_step_replay(self, U, dt=0.0, dt_out=None):

@@ -549,8 +549,8 @@ extern "C" int mpmc_rk_step_replay(mpmc_ctx* c, double* U, double dt, double* dt
   return check_launch(c, "rk_step_replay");
 }
 
-extern "C" int mpmc_rk_step_record(mpmc_ctx* c, double* U, double dt, uint32_t* tape, double* U_stages,
-                                   double* W_stages) {
+extern "C" int mpmc_rk_step_record_dt(mpmc_ctx* c, double* U, double dt, uint32_t* tape, double* U_stages,
+                                      double* W_stages, double* dt_out) {
   if (!c || !U || !U_stages) return fail(c, MPMC_INVALID_ARG, "rk_step_record: null argument");
   if (W_stages && c->precision != MPMC_FP64)
     return fail(c, MPMC_INVALID_ARG, "rk_step_record: W_stages needs an FP64 context");
@@ -565,7 +565,8 @@ extern "C" int mpmc_rk_step_record(mpmc_ctx* c, double* U, double dt, uint32_t* 
     return !W_stages || cudaMemcpyAsync(W_stages + k * nw, c->Wc, nw * sizeof(double), cudaMemcpyDeviceToDevice,
                                         s) == cudaSuccess;
   };
-  dt_gamma(c, c->rec, s, U, dt, -1.0, nullptr);
+  if (dt_out) cudaMemsetAsync(c->counter, 0, sizeof(int), s);
+  dt_gamma(c, c->rec, s, U, dt, -1.0, dt_out);
   if (!keep(0)) return fail(c, MPMC_CUDA_ERROR, "rk_step_record: cache copy");
   stage(c, c->rec, s, U, U, 1.0, 0.0, 1.0, U1, nullptr, tape);
   prim(c, c->rec, s, U1, nullptr);
@@ -576,6 +577,11 @@ extern "C" int mpmc_rk_step_record(mpmc_ctx* c, double* U, double dt, uint32_t* 
   stage(c, c->rec, s, U, U2, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0, U, nullptr, tape ? tape + 2 * nf : nullptr);
   c->faces_done += 3ull * c->nface_total;
   return check_launch(c, "rk_step_record");
+}
+
+extern "C" int mpmc_rk_step_record(mpmc_ctx* c, double* U, double dt, uint32_t* tape, double* U_stages,
+                                   double* W_stages) {
+  return mpmc_rk_step_record_dt(c, U, dt, tape, U_stages, W_stages, nullptr);
 }
 
 extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double* U_stages, const double* W_stages,

@@ -1,7 +1,8 @@
 // Mixed-precision kernels of the MPMC stage: reconstruction, face EOS,
 // HLLC, regularization and diffusion fluxes in FP32 with FP32 accumulation;
-// the cell p-T equilibrium inversion, the positivity-limiter pseudo-updates
-// and the conservative RK accumulation in FP64.
+// the cell p-T equilibrium inversion in float-float with FP64's result rounded
+// to FP32, the positivity-limiter pseudo-updates and the conservative RK
+// accumulation in FP64.
 //
 // Uniform fields stay exactly uniform: every stencil value is reconstructed
 // as its deviation from the face's left cell (W_j - W_i, zero where P, T, u
