@@ -3,7 +3,7 @@
 stages with the update fused in) of the 3D droplet field, 256^3 periodic
 cells, 4 species (two stiffened liquids, air, helium) in 2 phases, CDI and
 non-dilute diffusion on, on one GB300 per rank; the FP64 path and the mixed
-path (FP32 bulk, FP64 EOS inversion / positivity bounds / RK accumulation).
+path (FP32 bulk, float-float EOS inversion, FP64 positivity bounds / RK accumulation).
 
 One JSON line on rank 0:
   * `value`: device-timed cell-updates/s of the FP64 path (inputs resident
@@ -58,9 +58,9 @@ L2_BYTES = 129 * 2 ** 20
 TRAFFIC_GRID = 256
 TRAFFIC = {"k_face": 6.279e9, "mx::k_face": 3.762e9, "k_prim": 4.207e9, "mx::k_prim": 3.110e9,
            "k_update": 5.961e9, "mx::k_update": 5.958e9}
-TRAFFIC_SOURCES = ("paper_2504_14063_gb300/csrc/mpmc_kernels.cuh", "paper_2504_14063_gb300/csrc/mpmc_device.cuh",
-                   "paper_2504_14063_gb300/csrc/mpmc_kernels_d3.cu", "paper_2504_14063_gb300/csrc/mpmc_mixed.cuh",
-                   "paper_2504_14063_gb300/csrc/mpmc_mixed_d3.cu", "paper_2504_14063_gb300/csrc/mpmc_update.cuh")
+TRAFFIC_SOURCES = tuple("paper_2504_14063_gb300/csrc/" + f for f in (
+    "mpmc_kernels.cuh", "mpmc_device.cuh", "mpmc_ff.h", "mpmc_avg.h", "mpmc_fast.cuh", "mpmc_kernels_d3.cu",
+    "mpmc_fast_d3.cu", "mpmc_mixed.cuh", "mpmc_mixed_d3.cu", "mpmc_update.cuh"))
 TRAFFIC_SHA256 = "2fe30e2cc812f9f9efc25d643d0188eb8434e4643e20d8be13770ab9422f1c4d"
 
 
@@ -520,14 +520,15 @@ def fma_peaks(mp, torch, reps=5):
     return out
 
 
-def update_bytes(p, stage):
+def update_bytes(p, stage, flux_bytes=8):
     """Bytes the divergence + RK update kernel moves as designed for one
     launch: U^n (and U^(k) when distinct, stages 2 and 3), each face flux of
-    every direction once, and U^(k+1)."""
+    every direction once (flux_bytes each: 4 on the mixed path), and
+    U^(k+1)."""
     nv, D, N = p.nvars, p.dim, p.ncells
     faces = sum(N // p.n[d] * (p.n[d] + 1) for d in range(D))
     states = 2 if stage == 1 else 3
-    return 8 * nv * (states * N) + 8 * nv * faces
+    return 8 * nv * (states * N) + flux_bytes * nv * faces
 
 
 def update_flops(p, stage):
@@ -717,6 +718,7 @@ def main():
 
     n_w64 = cache_fields(p)
     upd_b = (update_bytes(p, 1) + 2 * update_bytes(p, 2)) / 3.0
+    upd_bm = (update_bytes(p, 1, 4) + 2 * update_bytes(p, 2, 4)) / 3.0
     upd_f = p.ncells * (update_flops(p, 1) + 2 * update_flops(p, 2)) / 3.0
 
     def update_roof(kernel, ms, note):
@@ -744,14 +746,19 @@ def main():
         "k_update": update_roof("k_update", kp["update"][0],
                                 "FP64 flux differences and RK combination; bytes and flops averaged over "
                                 "the three stages"),
-        "mx::k_update": update_roof("mx::k_update", kpm["update"][0], "the same body on the FP64 fluxes"),
+        "mx::k_update": hbm("mx::k_update", kpm["update"][0], upd_bm,
+                            "FP32 fluxes, differenced and summed in float-float, RK combination in FP64"),
     }
-    prim_note = ("bound by the FP64 pipe, not HBM: an ncu capture of the 128^3 case shows the FP64 pipe "
-                 "82-88 % active and DRAM at 2-4 % of peak; the iterative p-T solve has no fixed flop "
-                 "count, so the HBM fraction of the bytes it moves is what is reported")
-    rooflines["k_prim"] = hbm("k_prim", kp["prim"][0], prim_bytes(p, n_w64, 8), "FP64 p-T inversion; " + prim_note)
+    roofline["note"] = ("operations of the method as itemized; the interpolation's weights, the face average's "
+                        "scalars and the sound speed run in float-float on the FP32 pipe, so that the rate in "
+                        "these operations exceeds the FP64 pipe's")
+    prim_note = ("the iterative p-T solve has no fixed flop count, so the HBM fraction of the bytes it moves is "
+                 "what is reported")
+    rooflines["k_prim"] = hbm("k_prim", kp["prim"][0], prim_bytes(p, n_w64, 8),
+                              "p-T inversion iterated on the FP32 pipe, finished in FP64; " + prim_note)
     rooflines["mx::k_prim"] = hbm("mx::k_prim", kpm["prim"][0], prim_bytes(p, n_w64, 4),
-                                  "FP64 p-T inversion, FP32 cache; " + prim_note)
+                                  "float-float p-T inversion, FP32 cache (issue-bound: 63 % of the issue slots, "
+                                  "FP64 pipe 1 %, in an ncu capture at 128^3); " + prim_note)
     mixed = {"value": vm, "unit": UNIT, "ms_per_step": 1e3 * tm / args.steps, "speedup_vs_fp64": vm / value,
              "clocks": clk_m, "kernel_ms_per_step": {k: v[0] * v[1] for k, v in kpm.items()},
              "error_vs_fp64": err, "status": mstat}
