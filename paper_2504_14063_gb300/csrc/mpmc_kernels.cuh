@@ -738,8 +738,12 @@ __global__ void __launch_bounds__(FACE_THREADS)
 }
 
 // ---------------------------------------------------------------------------
+// Four blocks per SM (64 registers): all of a cell's loads in flight at once
+// took 144 registers and left 12 % of the warps (256^3 droplet field, per step
+// of three: 8.5 ms unbounded, 6.5 with three or four blocks; 1024 x 512 0.15
+// either way).  The FP64 pipe bounds it: 62 instructions per cell.
 template <int NS, int D>
-__global__ void __launch_bounds__(CELL_THREADS, 1)
+__global__ void __launch_bounds__(CELL_THREADS, 4)
     k_update(const KParams P, const double* __restrict__ Un, const double* __restrict__ Uk,
              const double* __restrict__ F0, const double* __restrict__ F1, const double* __restrict__ F2,
              const double* __restrict__ scal, const double rk0, const double rk1, const double rk2,
