@@ -56,12 +56,12 @@ L2_BYTES = 129 * 2 ** 20
 # and while the kernels' sources hash to the captured version (None
 # otherwise).
 TRAFFIC_GRID = 256
-TRAFFIC = {"k_face": 6.279e9, "mx::k_face": 3.762e9, "k_prim": 4.207e9, "mx::k_prim": 3.110e9,
-           "k_update": 5.961e9, "mx::k_update": 5.958e9}
+TRAFFIC = {"k_face": 9.706e9, "mx::k_face": 3.321e9, "k_prim": 4.260e9, "mx::k_prim": 3.190e9,
+           "k_update": 5.993e9, "mx::k_update": 4.294e9}
 TRAFFIC_SOURCES = tuple("paper_2504_14063_gb300/csrc/" + f for f in (
     "mpmc_kernels.cuh", "mpmc_device.cuh", "mpmc_ff.h", "mpmc_avg.h", "mpmc_fast.cuh", "mpmc_kernels_d3.cu",
     "mpmc_fast_d3.cu", "mpmc_mixed.cuh", "mpmc_mixed_d3.cu", "mpmc_update.cuh"))
-TRAFFIC_SHA256 = "2fe30e2cc812f9f9efc25d643d0188eb8434e4643e20d8be13770ab9422f1c4d"
+TRAFFIC_SHA256 = "967111c73c4347f68a056f8800f2232316c8c00d8f38ba94677b44d1558ed938"
 
 
 def sources_sha256():
