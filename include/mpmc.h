@@ -227,8 +227,11 @@ int mpmc_dt_gamma(mpmc_ctx* ctx, const double* U, double* out_dev);
  * Sec. 3.3.1 is differentiated on the branch the forward took, and dt and
  * Gamma (Sec. 3.4, Sec. 3.2) are frozen at the forward values.  A species
  * with Y_k = 0 exactly contributes no sensitivity (the forward omits it).
- * Adjoint scratch (cache adjoint, two state-sized buffers, one step of flags)
- * is allocated on the first call; MPMC_OUT_OF_MEMORY if that fails.
+ * Adjoint scratch (one direction's face slots, a cache adjoint, three
+ * state-sized buffers, one step of flags) is allocated on the first call;
+ * MPMC_OUT_OF_MEMORY if that fails.  The first mpmc_rk_step_adjoint without
+ * W_stages adds a second primitive cache (mpmc_cache_doubles) after it, kept
+ * with the context; without memory for it the step recomputes that cache.
  *
  * lam_U += (dL/dU)^T lam_dUdt for the stage of mpmc_rhs at U.  stage: as for
  * mpmc_rhs (nullable; dt <= 0 / Gamma < 0 are recomputed from U_n exactly as

@@ -27,7 +27,8 @@ struct mpmc_ctx {
   cudaStream_t cap;  // internal stream used only to capture graphs
   int device;
   double* Wc = nullptr;
-  double* Wc2 = nullptr;  // a second cache, for the reverse step (first use)
+  double* Wc2 = nullptr;  // a second cache, for the reverse step (first use without W_stages)
+  bool wc2_tried = false;
   double* F[3] = {nullptr, nullptr, nullptr};
   long long nface[3] = {0, 0, 0};
   long long nface_total = 0;
@@ -474,16 +475,30 @@ static int ensure_adjoint(mpmc_ctx* c) {
   long long nfmax = 0;
   for (int d = 0; d < P.dim; ++d) nfmax = c->nface[d] > nfmax ? c->nface[d] : nfmax;
   if (!c->Cslots) rc = alloc(c, (void**)&c->Cslots, (size_t)c->aops.slots(P) * nfmax * sizeof(double));
-  if (!rc && !c->Wc2 && cudaMalloc((void**)&c->Wc2, (size_t)P.nW * P.wstride * sizeof(double)) != cudaSuccess) {
-    cudaGetLastError();
-    c->Wc2 = nullptr;   // the reverse step then recomputes U^n's cache
-  }
   if (!rc && !c->gW) rc = alloc(c, (void**)&c->gW, (size_t)P.nW * P.wstride * sizeof(double));
   if (!rc && !c->gU) rc = alloc(c, (void**)&c->gU, st_bytes);
   if (!rc && !c->lamA) rc = alloc(c, (void**)&c->lamA, st_bytes);
   if (!rc && !c->lamB) rc = alloc(c, (void**)&c->lamB, st_bytes);
   if (!rc && !c->tape_int) rc = alloc(c, (void**)&c->tape_int, 3 * (size_t)c->nface_total * sizeof(uint32_t));
   return rc;
+}
+
+// The reverse step's second primitive cache, which it can do without: allocated
+// once everything that it needs is there, tried once (a later call could be
+// under capture), and not under a capture of the context's stream
+static void second_cache(mpmc_ctx* c) {
+  if (c->wc2_tried) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (cap != cudaStreamCaptureStatusNone) return;
+  c->wc2_tried = true;
+  if (cudaMalloc((void**)&c->Wc2, (size_t)c->P.nW * c->P.wstride * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    c->Wc2 = nullptr;   // U^n's cache is then recomputed
+  }
 }
 
 // face fluxes of one stage for their flags only (no divergence / update)
@@ -590,6 +605,7 @@ extern "C" int mpmc_rk_step_adjoint(mpmc_ctx* c, const double* U_n, const double
   if (W_stages && !U_stages) return fail(c, MPMC_INVALID_ARG, "rk_step_adjoint: W_stages without U_stages");
   int rc = ensure_adjoint(c);
   if (rc) return rc;
+  if (!W_stages) second_cache(c);
   const KParams& P = c->P;
   const long long nf = c->nface_total, n = (long long)P.nv * P.ncell;
   cudaStream_t s = c->stream;

@@ -1,0 +1,61 @@
+"""Device memory of the reverse passes: what they can do without is allocated
+only by the call that uses it and never in the place of what they need."""
+import pytest
+import torch
+
+from paper_2504_14063_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+MB2 = 2 << 20   # the driver's allocation granularity
+
+
+@pytest.fixture(scope="module")
+def mods():
+    from paper_2504_14063_gb300 import autograd, binding
+    return autograd, binding
+
+
+def _free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_second_cache_comes_last_and_only_where_it_is_used(mods):
+    _, mp = mods
+    p = W.random_smooth_2d(nx=640, ny=640, seed=3)
+    ctx = mp.Context(p)
+    U0 = ctx.init_state(torch.from_numpy(p.prim))
+    lam = torch.randn(U0.shape, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(0))
+    dt = 0.5 * float(ctx.dt_gamma(U0)[0])
+    tape = torch.empty(3 * ctx.nfaces_total, dtype=torch.int32, device="cuda")
+    caches = torch.empty(3 * ctx.cache_doubles, dtype=torch.float64, device="cuda")
+    stages = ctx.rk_step_record(U0.clone(), dt, tape, None, caches)
+    out, ref, lamW = torch.empty_like(U0), torch.zeros_like(U0), torch.zeros_like(ctx.primitives(U0))
+    cache = 8 * ctx.cache_doubles
+    assert cache > 16 * MB2
+    a = _free()
+    ctx.rhs_adjoint(U0, None, None, lam, out)
+    b = _free()
+    ctx.primitives_adjoint(U0, lamW, out)
+    ctx.rk_step_adjoint(U0, lam, dt, tape, out, stages, caches)
+    assert _free() == b        # neither takes the cache that it has no use for
+    ctx.rk_step_adjoint(U0, lam, dt, tape, ref, stages)
+    c = _free()
+    assert cache <= b - c <= cache + MB2
+    need = a - b               # what the reverse step cannot do without
+    # a context with room for that and half a cache
+    tight = mp.Context(p)
+    left = need + cache // 2
+    fill = torch.empty(_free() - left, dtype=torch.uint8, device="cuda")
+    try:
+        assert need < _free() < need + cache
+        tight.rk_step_adjoint(U0, lam, dt, tape, out, stages)
+        torch.cuda.synchronize()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert torch.equal(out, ref)
+    # (and the attempt is not repeated once there is room)
+    d = _free()
+    tight.rk_step_adjoint(U0, lam, dt, tape, out, stages)
+    assert _free() == d and torch.equal(out, ref)
