@@ -20,7 +20,8 @@ pass are replayed and each step's dt and Gamma are frozen (Sec. 3.3, 3.4).
         and limiter flags) and sweeps it in reverse, so memory holds the
         checkpoints plus one segment of inputs, stage states and flags.  The
         last segment, which the backward pass takes first, is recorded by the
-        forward pass itself where it fits in an eighth of the free memory.
+        forward pass itself where it fits in an eighth of the free memory, which
+        the graph then holds until the backward pass.
 """
 import torch
 
@@ -151,15 +152,24 @@ class _Rollout(torch.autograd.Function):
         if probe is not None and gJ != 0.0:
             lamW = torch.zeros((len(ctx.prim_fields),) + tuple(lam.shape[1:]), dtype=torch.float64,
                                device=lam.device)
+        bufs = None
         for seg in reversed(range(len(fctx.ckpts))):
             k0, k1 = seg * every, min(n, (seg + 1) * every)
             m = k1 - k0
             if fctx.kept is not None and seg == len(fctx.ckpts) - 1:
-                states, stages, tapes, wst = fctx.kept
+                bufs = fctx.kept
                 fctx.kept = None   # (another backward pass replays it)
+                states, stages, tapes, wst = bufs
             else:
-                # replay the segment, keeping every step's input, stage states and flags
-                states, stages, tapes, wst = _segment(ctx, m, lam)
+                # replay the segment, keeping every step's input, stage states and
+                # flags, in the buffers of the one before (one segment's memory)
+                if bufs is not None and bufs[1].shape[0] < m:
+                    bufs = states = stages = tapes = wst = None
+                if bufs is None:
+                    bufs = _segment(ctx, m, lam)
+                elif bufs[3] is None:
+                    bufs = bufs[:3] + (_stage_caches(ctx, bufs[1].shape[0], lam.device),)
+                states, stages, tapes, wst = bufs
                 states[0].copy_(fctx.ckpts[seg])
                 for q in range(m):
                     states[q + 1].copy_(states[q])

@@ -59,3 +59,35 @@ def test_second_cache_comes_last_and_only_where_it_is_used(mods):
     d = _free()
     tight.rk_step_adjoint(U0, lam, dt, tape, out, stages)
     assert _free() == d and torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("n,every", [(12, 4), (10, 4), (9, 9)])
+@pytest.mark.parametrize("kept", [False, True])
+def test_backward_of_a_rollout_holds_one_segment(mods, monkeypatch, n, every, kept):
+    """The backward pass allocates no more than one segment's buffers, kept or
+    not, whole or with a shorter last one (measured in torch's allocator, which
+    every buffer of it comes from)."""
+    ag, mp = mods
+    p = W.shock_bubble_2d(nx=256, ny=128, seed=1)
+    ctx = mp.Context(p)
+    prim = torch.from_numpy(p.prim).cuda().requires_grad_()
+    probe = torch.zeros(p.prim.shape[1:], dtype=torch.float64, device="cuda")
+    probe[:, :, 80] = 1.0 / 128
+    seg = ag._segment
+    if not kept:
+        monkeypatch.setattr(ag, "_segment", lambda c, m, like, share=None: None if share is not None else seg(c, m, like))
+    state = ctx.nv * ctx.ncells * 8
+    one = (3 * every + 1) * state + every * 3 * (ctx.nfaces_total * 4 + ctx.cache_doubles * 8)
+    U, J, _ = ag.rollout(ctx, ag.init_state(ctx, prim), n, every=every, probe=probe)
+    torch.cuda.synchronize()
+    base = torch.cuda.memory_allocated()
+    torch.cuda.reset_peak_memory_stats()
+    g, = torch.autograd.grad(J, prim)
+    assert float(g.abs().max()) > 0
+    peak = torch.cuda.max_memory_allocated() - base
+    print(f"peak {peak / one:.2f} segments")
+    # besides the segment: the adjoint, its copies, the probe's field adjoint
+    # and the gradient, a few fields of a cell each
+    rest = 12 * state
+    assert peak <= (0 if kept and n % every == 0 else one) + rest
+    assert rest < 0.5 * one
