@@ -190,13 +190,17 @@ int mpmc_init_state(mpmc_ctx* ctx, const double* prim, double* U);
  * limiter is stage-aware (Sec. 3.3.2): stage = NULL means a forward-Euler
  * stage from U with the CFL step and Gamma of U.  dUdt: device, same layout
  * as U.  flags (nullable, device): per face, all faces of direction 0, then
- * 1, then 2, each laid out like cells with n[d]+1 entries along d. */
+ * 1, then 2, each laid out like cells with n[d]+1 entries along d.  With
+ * flags the call runs in the arithmetic that mpmc_rhs_adjoint recomputes in
+ * (dUdt, dt and Gamma then differ from the call's without flags by rounding,
+ * and it takes about twice as long). */
 int mpmc_rhs(mpmc_ctx* ctx, const double* U, double* dUdt, const mpmc_stage* stage, uint32_t* flags);
 
 /* One SSP-RK3 step (Eq. SSPRK3) in place on device array U.  dt > 0: fixed
  * step; dt <= 0: CFL step (Sec. 3.4) from U^n computed on the device.  tape
  * (nullable, device, 3 x faces uint32): per stage and face the flag bits
- * above, for replay by the adjoint. */
+ * above, for replay by the adjoint; with it the step is, bit for bit, the one
+ * of mpmc_rk_step_record (without it, it rounds otherwise and is faster). */
 int mpmc_rk_step(mpmc_ctx* ctx, double* U, double dt, uint32_t* tape);
 
 /* n SSP-RK3 steps in place (replayed as a CUDA graph); each step takes its
@@ -235,8 +239,8 @@ int mpmc_dt_gamma(mpmc_ctx* ctx, const double* U, double* out_dev);
  *
  * lam_U += (dL/dU)^T lam_dUdt for the stage of mpmc_rhs at U.  stage: as for
  * mpmc_rhs (nullable; dt <= 0 / Gamma < 0 are recomputed from U_n exactly as
- * the forward did); tape: that call's flags (nullable: the decisions are
- * recomputed); lam_dUdt, lam_U: device, layout of U. */
+ * mpmc_rhs with flags did); tape: that call's flags (nullable: the decisions
+ * are recomputed as it takes them); lam_dUdt, lam_U: device, layout of U. */
 int mpmc_rhs_adjoint(mpmc_ctx* ctx, const double* U, const mpmc_stage* stage, const uint32_t* tape,
                      const double* lam_dUdt, double* lam_U);
 
@@ -253,15 +257,16 @@ int mpmc_rk_step_record_dt(mpmc_ctx* ctx, double* U, double dt, uint32_t* tape, 
                            double* dt_out);
 
 /* One SSP-RK3 step in place in the arithmetic of mpmc_rk_step_record (bit for
- * bit the states that it records; mpmc_rk_step and mpmc_step_n round
- * otherwise): the forward step of a differentiated run.  dt as for
+ * bit the states that it records; mpmc_rk_step without a tape and mpmc_step_n
+ * round otherwise): the forward step of a differentiated run.  dt as for
  * mpmc_rk_step; dt_out (nullable, device double) receives the step's length. */
 int mpmc_rk_step_replay(mpmc_ctx* ctx, double* U, double dt, double* dt_out);
 
 /* Reverse of one SSP-RK3 step (Eq. SSPRK3) from U_n:
  *   lam_n = (dU^{n+1}/dU^n)^T lam_next.
- * dt: as passed to mpmc_rk_step_record (<= 0: the CFL step of U_n, recomputed
- * bit-identically).  U_stages (nullable): the step's stage states from
+ * dt: as passed to mpmc_rk_step_record, mpmc_rk_step_replay or mpmc_rk_step
+ * with a tape (<= 0: the CFL step of U_n, recomputed bit-identically to
+ * theirs).  U_stages (nullable): the step's stage states from
  * mpmc_rk_step_record; recomputed from U_n when null.  W_stages (nullable;
  * only with U_stages): that call's primitive caches, used instead of
  * recomputing them (the result is the same bit for bit).  tape: that step's

@@ -209,7 +209,9 @@ class Context:
         return U
 
     def rhs(self, U, dUdt=None, stage=None, flags=None):
-        """stage: None or dict(U_n=tensor, rk=(rk0, rk1, rk2), dt=float, Gamma=float)."""
+        """stage: None or dict(U_n=tensor, rk=(rk0, rk1, rk2), dt=float, Gamma=float).
+        flags (int32 of nfaces_total): the limiter decisions, for rhs_adjoint; with
+        them the call runs in its arithmetic (slower, equal to rounding)."""
         dUdt = torch.empty_like(U) if dUdt is None else dUdt
         sp = None
         if stage is not None:
@@ -223,6 +225,9 @@ class Context:
         return dUdt
 
     def rk_step(self, U, dt=0.0, tape=None):
+        """One SSP-RK3 step in place.  tape (int32 of 3 x nfaces_total): the limiter
+        decisions, for rk_step_adjoint; with it the step is rk_step_record's bit
+        for bit (slower, equal to rounding)."""
         self._check(lib.mpmc_rk_step(self.h, _dev(U), float(dt), _ptr(tape)))
         return U
 

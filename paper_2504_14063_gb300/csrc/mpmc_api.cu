@@ -20,7 +20,7 @@ static constexpr int NFAM_MAX = 6;
 struct mpmc_ctx {
   KParams P;
   Ops ops;
-  Ops rec;   // the recording calls' kernels (FP64: plain FP64 arithmetic; else ops)
+  Ops rec;   // the kernels of calls with a tape or flags, and of the adjoint's (FP64: plain FP64 arithmetic; else ops)
   AdjOps aops;
   int precision;
   cudaStream_t stream;
@@ -382,18 +382,21 @@ extern "C" int mpmc_rhs(mpmc_ctx* c, const double* U, double* dUdt, const mpmc_s
   const double rk0 = st ? st->rk0 : 1.0, rk1 = st ? st->rk1 : 0.0, rk2 = st ? st->rk2 : 1.0;
   const double dt = st ? st->dt : 0.0, G = st ? st->Gamma : -1.0;
   cudaStream_t s = c->stream;
+  // flags are for mpmc_rhs_adjoint: with them, the arithmetic that it recomputes in
+  const Ops& ops = flags ? c->rec : c->ops;
   // dt / Gamma from U^n (always run so that the prim pass of U_n also
   // validates it); then the primitive cache of U
-  dt_gamma(c, c->ops, s, Un, dt, G, nullptr);
-  if (Un != U) prim(c, c->ops, s, U, nullptr);
-  stage(c, c->ops, s, Un, U, rk0, rk1, rk2, nullptr, dUdt, flags);
+  dt_gamma(c, ops, s, Un, dt, G, nullptr);
+  if (Un != U) prim(c, ops, s, U, nullptr);
+  stage(c, ops, s, Un, U, rk0, rk1, rk2, nullptr, dUdt, flags);
   c->faces_done += c->nface_total;
   return check_launch(c, "rhs");
 }
 
 extern "C" int mpmc_rk_step(mpmc_ctx* c, double* U, double dt, uint32_t* tape) {
   if (!c || !U) return fail(c, MPMC_INVALID_ARG, "rk_step: null argument");
-  rk3(c, c->ops, c->stream, U, dt, tape, nullptr);
+  // a tape is for mpmc_rk_step_adjoint: with it, the arithmetic that it recomputes in
+  rk3(c, tape ? c->rec : c->ops, c->stream, U, dt, tape, nullptr);
   c->faces_done += 3ull * c->nface_total;
   return check_launch(c, "rk_step");
 }
@@ -544,7 +547,7 @@ extern "C" int mpmc_rhs_adjoint(mpmc_ctx* c, const double* U, const mpmc_stage* 
   const double rk0 = st ? st->rk0 : 1.0, rk1 = st ? st->rk1 : 0.0, rk2 = st ? st->rk2 : 1.0;
   const double dt = st ? st->dt : 0.0, G = st ? st->Gamma : -1.0;
   cudaStream_t s = c->stream;
-  // the same dt / Gamma and primitive cache as mpmc_rhs
+  // the same dt / Gamma and primitive cache as mpmc_rhs with flags
   dt_gamma(c, c->rec, s, Un, dt, G, nullptr);
   if (Un != U) prim(c, c->rec, s, U, nullptr);
   if (!tape) {

@@ -8,9 +8,10 @@
 // The right-hand sides' error against extended precision went from 1 to
 // 0.5 .. 1.1 of the FP64 form's (four workloads, every field).
 //
-// Steps and right-hand sides run these kernels.  The recording calls of the
-// discrete adjoint (mpmc_rk_step_record and what mpmc_rk_step_adjoint and
-// mpmc_rhs_adjoint recompute) run mpmc_kernels.cuh's: the reverse sweep
+// Steps and right-hand sides run these kernels, unless they return limiter
+// flags for a reverse pass.  Those, the recording calls of the discrete adjoint
+// (mpmc_rk_step_record, mpmc_rk_step_replay) and what mpmc_rk_step_adjoint and
+// mpmc_rhs_adjoint recompute run mpmc_kernels.cuh's: the reverse sweep
 // evaluates the faces in that form, and the derivative it takes is
 // discontinuous in the states' rounding (the mass-fraction limiter acts
 // unless sum Y is one to 1e-15, a stencil of rounding noise has weights of
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(SPLIT ? 32 * SPLIT_WARPS<NS, D> : FACE_THREADS
     k_face(const __grid_constant__ KParams P, const double* __restrict__ Wc, const double* __restrict__ Un,
            const double* __restrict__ Uk, const double* __restrict__ Uin, const double* __restrict__ scal,
            const double rk0, const double rk1, const double rk2, double* __restrict__ F,
-           uint32_t* __restrict__ flags, unsigned long long* __restrict__ stats) {
+           unsigned long long* __restrict__ stats) {
   constexpr int NV = NS + D + 1;
   constexpr int d = DIR;
   const int f0 = P.n[0] + (d == 0), f1 = P.n[1] + (d == 1), f2 = P.n[2] + (d == 2);
@@ -1052,7 +1053,6 @@ __global__ void __launch_bounds__(SPLIT ? 32 * SPLIT_WARPS<NS, D> : FACE_THREADS
 
 #pragma unroll
   for (int v = 0; v < NV; ++v) F[(long long)v * nf + fid] = Fx[v];
-  if (flags) flags[fid] = fl;
   if (stats && fl) {
     if (fl & F_HLLC_FALLBACK) atomicAdd(stats + 1, 1ull);
     if (fl & F_CDI_DROPPED) atomicAdd(stats + 2, 1ull);
@@ -1075,7 +1075,7 @@ template <int NS, int D, int RC>
 struct FaceImpl {
   static void face(const KParams& P, cudaStream_t s, int d, const double* Wc, const double* Un, const double* Uk,
                    const double* Uin, const double* scal, double rk0, double rk1, double rk2, double* F,
-                   uint32_t* flags, unsigned long long* stats) {
+                   uint32_t* /*flags: the recording kernels'*/, unsigned long long* stats) {
     long long nf = 1;
     for (int e = 0; e < 3; ++e) nf *= (long long)(P.n[e] + (e == d));
     if constexpr (D < 3) {
@@ -1086,23 +1086,23 @@ struct FaceImpl {
         constexpr int nt = 32 * SPLIT_WARPS<NS, D>;
         if (d == 0)
           fast::k_face<NS, D, 0, RC, true><<<nblocks(nf, 32), nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
-                 flags, stats);
+                 stats);
         else
           fast::k_face<NS, D, (D > 1 ? 1 : 0), RC, true><<<nblocks(nf, 32), nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal,
-                 rk0, rk1, rk2, F, flags, stats);
+                 rk0, rk1, rk2, F, stats);
         return;
       }
     }
     const int nt = block_threads(nf, FACE_THREADS);
     const unsigned nb = nblocks(nf, nt);
     if (d == 0)
-      fast::k_face<NS, D, 0, RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F, flags, stats);
+      fast::k_face<NS, D, 0, RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F, stats);
     else if (d == 1)
       fast::k_face<NS, D, (D > 1 ? 1 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
-                                                                     flags, stats);
+                                                                     stats);
     else
       fast::k_face<NS, D, (D > 2 ? 2 : 0), RC><<<nb, nt, 0, s>>>(P, Wc, Un, Uk, Uin, scal, rk0, rk1, rk2, F,
-                                                                     flags, stats);
+                                                                     stats);
   }
 };
 
