@@ -20,6 +20,8 @@
 #include <cstdint>
 #include <cstring>
 
+#include "mpmc_narrow.h"
+
 #ifdef __CUDACC__
 #define MPMC_FF __host__ __device__ __forceinline__
 #else
@@ -193,6 +195,32 @@ MPMC_FF double ff_widen(float f, int E) {
   const uint32_t b = fbits(f), e = (b >> 23) & 0xffu;
   const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((uint32_t)(E - 127) << 20));
   return e ? dmake(hi, b << 29) : 0.0;
+}
+
+// sum_d (a_d - b_d) of FP32 numbers to FP64 rounding: the differences are exact
+// as pairs, their high parts are summed exactly, and what that leaves is summed
+// as a pair (within 2^-64 of the differences' magnitudes).  One rounding of the
+// sum follows, where FP64 differences and sums take 2 D - 1.
+// ok: false where a part leaves FP32's normal range; the caller takes FP64.
+template <int D>
+MPMC_FF double ff_diff_sum(const float* a, const float* b, bool& ok) {
+  ff s = ff_two(a[0], -b[0]);
+  if (D == 1) {
+    ok = ok && widens(s.h) && widens(s.l);
+    return widen(s.h) + widen(s.l);
+  }
+  ff r = {s.l, 0.f};
+#pragma unroll
+  for (int d = 1; d < D; ++d) {
+    const ff t = ff_two(a[d], -b[d]);
+    s = ff_two(s.h, t.h);
+    ff q = ff_two(r.h, s.l);
+    r = ff{q.h, fadd(r.l, q.l)};
+    q = ff_two(r.h, t.l);
+    r = ff{q.h, fadd(r.l, q.l)};
+  }
+  ok = ok && widens(s.h) && widens(r.h) && widens(r.l);
+  return widen(s.h) + (widen(r.h) + widen(r.l));
 }
 
 // ---------------------------------------------------------------------------

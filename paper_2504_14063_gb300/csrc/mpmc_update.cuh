@@ -1,8 +1,8 @@
 // Divergence of the face fluxes (Eq. DiscreteGoverningEquations) and the
 // SSP-RK combination (Eq. SSPRK3) of one cell, from face fluxes F_d[v][face]
 // of type FT: double, or float on the mixed path (every flux enters its two
-// cells with the same value, so that the sum over cells telescopes to the
-// rounding of the combination).
+// cells with the same value, and its cells' sums are FP64's, so that the sum
+// over cells telescopes to FP64 rounding).
 #pragma once
 #include "mpmc_device.cuh"
 
@@ -20,12 +20,14 @@ __device__ __forceinline__ void flux_sums(const double* const* Fd, const long lo
   }
 }
 
-// the same of FP32 fluxes: the differences exactly as float-floats, their sum
-// to 2^-47 of the largest, on the FP32 pipe.  (FP64 differences and sums, on
-// fluxes widened by the face pass, were 5 of the update's 8 FP64 operations
-// per component in 3D, and twice the flux traffic.)  Sums beyond FP32's normal
-// range take FP64, once all are formed: a branch per component would keep the
-// next one's loads back.
+// the same of FP32 fluxes: the differences and all but the last two additions
+// on the FP32 pipe (ff_diff_sum).  (FP64 differences and sums, on fluxes widened
+// by the face pass, were 5 of the update's 8 FP64 operations per component in
+// 3D, and twice the flux traffic.  With one FP64 addition, of a pair that holds
+// the sum to 2^-47 of the largest difference, a 256^3 step takes 46.2 ms for 47.0,
+// but its cells no longer telescope to FP64 rounding.)  Sums beyond FP32's normal range take FP64,
+// once all are formed: a branch per component would keep the next one's loads
+// back.
 template <int NV, int D>
 __device__ __forceinline__ void flux_sums(const float* const* Fd, const long long* nf, const long long* fm,
                                           const long long* fp, double* fs) {
@@ -37,16 +39,10 @@ __device__ __forceinline__ void flux_sums(const float* const* Fd, const long lon
       a[v][d] = Fd[d][(long long)v * nf[d] + fm[d]];
       b[v][d] = Fd[d][(long long)v * nf[d] + fp[d]];
     }
-  bool general = false;
+  bool ok = true;
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    ff s = ff_two(a[v][0], -b[v][0]);
-#pragma unroll
-    for (int d = 1; d < D; ++d) s = ff_add(s, ff_two(a[v][d], -b[v][d]));
-    general = general || !widens(s.h) || !widens(s.l);
-    fs[v] = widen(s.h) + widen(s.l);
-  }
-  if (general) {
+  for (int v = 0; v < NV; ++v) fs[v] = ff_diff_sum<D>(a[v], b[v], ok);
+  if (!ok) {
 #pragma unroll 1
     for (int v = 0; v < NV; ++v) {
       double f = (double)Fd[0][(long long)v * nf[0] + fm[0]] - (double)Fd[0][(long long)v * nf[0] + fp[0]];
