@@ -416,12 +416,12 @@ struct CellF {
   int st;
 };
 
-// an FP64 value that ff_of splits exactly as narrow rounds it: in 2^-126 ..
-// 2^125 or zero, and not half way between two FP32 numbers (ff_of takes ties
-// away from zero)
+// an FP64 value that ff_of splits with its low part, and whose high part is as
+// narrow rounds it: in 2^-74 .. 2^125 or zero, and not half way between two FP32
+// numbers (ff_of takes ties away from zero)
 __device__ __forceinline__ bool in_f32(double x) {
   const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu, l = (unsigned)__double2loint(x);
-  return (m - (897u << 20) < (251u << 20) && (l & 0x1fffffffu) != 0x10000000u) || (m | l) == 0u;
+  return (m - (949u << 20) < (199u << 20) && (l & 0x1fffffffu) != 0x10000000u) || (m | l) == 0u;
 }
 
 // a rounded to FP32; unsure: the bits below it come within `err` (relative to
@@ -464,12 +464,20 @@ __device__ __noinline__ void cell_fp64(const KParams& P, const double* __restric
 //   f(x) = sum_k w_k / (x + Pinf_k) - Cv,  w_k = Y_k R_k (E' - Pinf_k)
 // (NASG_T1 = NASG_T2) starts at the FP32 root of the quadratic with the
 // liquids merged into one, iterated in FP32 where they differ, and takes
-// Halley steps in float-float until one is below 1e-5 of the distance to the
-// nearest pole: what it leaves is of order 1e-15 of that distance.  The
-// rounding of a stiff liquid's terms leaves P within 2^-43 of the sum of their
-// magnitudes over the slope, a hundredth of P's FP32 rounding at P = 1e-4
-// Pinf; a result that comes that close to a rounding boundary is refused, so
-// that the FP32 cache holds what FP64 gives.  False (nothing written) there,
+// Halley steps with a float-float residual until one is below 1e-5 of the
+// distance to the nearest pole (what it leaves is of order 1e-15 of that
+// distance) and its own FP32 rounding below the residual's.  That leaves P
+// within 2^-44 of the sum of the terms' magnitudes over the slope, each term
+// taken before its cancellations (E' - Pinf; in fast flow E / rho against
+// |u|^2 / 2; e - q and v - b of a NASG liquid): a tenth of P's FP32 rounding for
+// a stiff liquid at P = 1e-4 Pinf.  A result that comes that close to a rounding
+// boundary is refused, T's margin widened alike, so that the FP32 cache holds
+// the FP64 root's rounding: in each of 3e7 random cells, of which 2 to 4 % are
+// refused at low speed.  (With 2^-43 of the terms after cancellation and no
+// bound on the step, 1 cell in 400 of flow at 30 times the thermal energy and 1
+// in 2e5 with two liquids had another P.  The FP64 form's solve of several
+// liquids stops 1e-12 of the pole's distance from the root: 1 in 1e5 of its own
+// P are one bit off.)  False (nothing written) there,
 // where the steps do not settle, and where a quantity leaves the range.
 template <int NS, int D>
 __device__ __forceinline__ bool cell_ff(const KParams& P, const ff* U, CellF<NS>& o) {
@@ -484,15 +492,25 @@ __device__ __forceinline__ bool cell_ff(const KParams& P, const ff* U, CellF<NS>
     u[d] = ff_mul(U[NS + d], v);
     ke = ff_addp(ke, ff_sqr(u[d]));
   }
-  ff em = ff_sub(ff_mul(U[NS + D], v), ff_mulf(ke, 0.5f)), vm = v, Cv = {0.f, 0.f};
+  const ff et = ff_mul(U[NS + D], v);
+  ff em = ff_sub(et, ff_mulf(ke, 0.5f)), vm = v, Cv = {0.f, 0.f};
+  float ae = fabsf(et.h) + 0.5f * ke.h, av = v.h;   // magnitudes of em's and vm's terms
   float pmin = 3e38f, pl = -1.f, Rg = 0.f, Rl = 0.f, wpl = 0.f;
   bool multi = false;
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     Y[k] = ff_mul(U[k], v);
     Cv = ff_add(Cv, ff_mul(Y[k], P.sff[k].cv));
-    if (P.has_q) em = ff_sub(em, ff_mul(Y[k], P.sff[k].q));
-    if (P.has_b) vm = ff_sub(vm, ff_mul(Y[k], P.sff[k].b));
+    if (P.has_q) {
+      const ff t = ff_mul(Y[k], P.sff[k].q);
+      em = ff_sub(em, t);
+      ae += fabsf(t.h);
+    }
+    if (P.has_b) {
+      const ff t = ff_mul(Y[k], P.sff[k].b);
+      vm = ff_sub(vm, t);
+      av += fabsf(t.h);
+    }
     if (Y[k].h > 0.f) {
       const float pk = P.f32.pinf[k], yr = Y[k].h * P.f32.Rk[k];
       pmin = fminf(pmin, pk);
@@ -508,15 +526,19 @@ __device__ __forceinline__ bool cell_ff(const KParams& P, const ff* U, CellF<NS>
   }
   if (!(em.h > 0.f && vm.h > 0.f)) return false;
   const ff Ep = P.has_b ? ff_mul(em, ff_rcp(vm)) : ff_mul(em, rho);
+  // what cancellation in em and vm multiplies their relative errors by (1
+  // without); of E' both
+  const float ce = ae * frcp(em.h), cE = ce + av * frcp(vm.h) - 1.f;
   // (a species with Y <= 0 enters as in pt_equilibrium: with several liquids
   // where Y is not zero, not otherwise)
   ff w[NS];
-  float wf[NS];
+  float wf[NS], wm[NS];   // wm: magnitudes of w's terms, with E' cancellation
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const bool on = multi ? Y[k].h != 0.f : Y[k].h > 0.f;
     w[k] = on ? ff_mul(ff_mul(Y[k], P.sff[k].R), ff_sub(Ep, P.sff[k].pinf)) : ff{0.f, 0.f};
     wf[k] = w[k].h;
+    wm[k] = on ? fabsf(Y[k].h * P.f32.Rk[k]) * (cE * Ep.h + P.f32.pinf[k]) : 0.f;
   }
   const float lo = -pmin;
   float x0;
@@ -540,20 +562,23 @@ __device__ __forceinline__ bool cell_ff(const KParams& P, const ff* U, CellF<NS>
       const ff r = ff_rcp(ff_add(x, P.sff[k].pinf)), t = ff_mul(w[k], r);
       const float tr = t.h * r.h;
       f = ff_add(f, t);
-      mag += fabsf(t.h);
+      mag += wm[k] * fabsf(r.h);
       df -= tr;
       d2 += tr * r.h;
     }
     const float g = frcp(df), s = f.h * g, dx = -s * frcp(1.f - s * (d2 * g));
-    err = 1.1e-13f * mag * fabsf(g);
-    done = fabsf(dx) <= 1e-5f * (x.h - lo);
+    // rounding of f, and of the step itself (FP32: 2^-21 of it)
+    const float ef = 5.7e-14f * mag * fabsf(g), ex = 4.8e-7f * fabsf(dx);
+    err = ef + ex;
+    done = fabsf(dx) <= 1e-5f * (x.h - lo) && ex <= 2.f * ef;
     x = ff_add(x, ff{dx, 0.f});
   }
   if (!done || !(fabsf(x.h) < 1e18f && x.h > lo)) return false;
   constexpr float E = 1.f / 65536.f;   // 2^-41 of a value
   bool unsure = false;
   const float p = ff_round(x, 0.f, unsure);
-  unsure = unsure || fabsf(x.l) + err > __uint_as_float(__float_as_uint(p) & 0x7f800000u) * 5.9604645e-8f;
+  // (NaN: unsure)
+  unsure = unsure || !(fabsf(x.l) + err <= __uint_as_float(__float_as_uint(p) & 0x7f800000u) * 5.9604645e-8f);
   float Yf[NS], T;
 #pragma unroll
   for (int k = 0; k < NS; ++k) Yf[k] = ff_round(Y[k], E, unsure);
@@ -568,15 +593,17 @@ __device__ __forceinline__ bool cell_ff(const KParams& P, const ff* U, CellF<NS>
                             : __fdividef(p + P.f32.gam[k] * P.f32.pinf[k], p + P.f32.pinf[k]);
         den += Yf[k] * P.f32.cv[k] * r;
       }
-    T = __fdividef(ff_round(em, E, unsure), den);
+    T = __fdividef(ff_round(em, E * ce, unsure), den);
   } else {
-    // T = (e - q) / (Cv + sum_k Y_k R_k Pinf_k / (P + Pinf_k))
+    // T = (e - q) / (Cv + sum_k Y_k R_k Pinf_k / (P + Pinf_k)); P's error moves it
+    // by at most err over the distance to the pole (in half ulps: times 2^25)
+    const float eT = 3.4e7f * err * frcp(x.h - lo);
     ff den = Cv;
 #pragma unroll
     for (int k = 0; k < NS; ++k)
       if (Y[k].h != 0.f && P.f32.pinf[k] > 0.f)
         den = ff_add(den, ff_mul(ff_mul(Y[k], P.sff[k].R), ff_mul(P.sff[k].pinf, ff_rcp(ff_add(x, P.sff[k].pinf)))));
-    T = ff_round(ff_mul(em, ff_rcp(den)), E, unsure);
+    T = ff_round(ff_mul(em, ff_rcp(den)), E * ce + eT, unsure);
   }
   if (!(fabsf(T) < 1e18f)) return false;
   float uf[3];

@@ -24,10 +24,10 @@ __device__ __forceinline__ void flux_sums(const double* const* Fd, const long lo
 // on the FP32 pipe (ff_diff_sum).  (FP64 differences and sums, on fluxes widened
 // by the face pass, were 5 of the update's 8 FP64 operations per component in
 // 3D, and twice the flux traffic.  With one FP64 addition, of a pair that holds
-// the sum to 2^-47 of the largest difference, a 256^3 step takes 46.2 ms for 47.0,
-// but its cells no longer telescope to FP64 rounding.)  Sums beyond FP32's normal range take FP64,
-// once all are formed: a branch per component would keep the next one's loads
-// back.
+// the sum to 2^-47 of the largest difference, a 256^3 step takes 46.2 ms for
+// 47.0, but its cells no longer telescope to FP64 rounding.)  Sums beyond FP32's
+// normal range take FP64, once all are formed: a branch per component would
+// keep the next one's loads back.
 template <int NV, int D>
 __device__ __forceinline__ void flux_sums(const float* const* Fd, const long long* nf, const long long* fm,
                                           const long long* fp, double* fs) {
