@@ -16,7 +16,7 @@
 //             = dT sum cv_k m_kj + sum R_k h_k + |du|^2 rho_i rho_j / (2 (rho_i + rho_j)),
 // the second linear (the kinetic energy that the average loses appears as
 // heat), so that y follows from x and the first is a rational function of x:
-// Newton steps, first in FP32, then two in float-float.  At its root
+// Newton steps, first in FP32, then two or three in float-float.  At its root
 //   X = T s_1 / sum cp_k M_k,  c^2 = (sum cp_k M_k) (sum M_k) / (T (s_2 sum cp_k M_k - s_1^2)),
 //   s_q = sum R_k M_k r_k^q,
 // which are Eq. SpeedOfSound and Appendix A's X with alpha and beta put in.
@@ -49,8 +49,11 @@ MPMC_FF ff ff_sqrt(ff a) {
 
 // X, c and 1 / c of the face between the cells i and j (mi, mj: partial
 // densities; ui, uj: velocities as the face sees them).  False (nothing
-// written) where the steps do not settle or a quantity leaves 2^-60..2^60:
-// the caller takes the FP64 form.
+// written) where the steps do not settle, where the jump's rounding would reach
+// 2^-41 of c (strong jumps of a liquid with traces of gas, whose pressure is
+// what they leave of it: FP64's own error is less there, elsewhere more or
+// both are below it), or where a quantity leaves 2^-60..2^60: the caller takes
+// the FP64 form.
 template <int NS, int D>
 MPMC_FF bool face_avg_ff(const SpeciesFF* sp, const double* mi, const double* mj, const double Pi, const double Pj,
                          const double Ti, const double Tj, const double* ui, const double* uj, double& X, double& c,
@@ -90,15 +93,19 @@ MPMC_FF bool face_avg_ff(const SpeciesFF* sp, const double* mi, const double* mj
   const ff Mt = ff_add(ri, rj);
   c0 = ff_add(c0, ff_mul(ff_mulf(u2, 0.5f), ff_mul(ff_mul(ri, rj), ff_rcp(Mt))));
   const ff inv = ff_rcp(cpM), y0 = ff_mul(c0, inv), y1 = ff_mul(gR, inv);
+  float am[NS], bm[NS];   // magnitudes of al's and be's terms
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
+    am[k] = fabs_(sp[k].R.h) * (fabs_(M[k].h * y0.h) + fabs_(al[k].h));
+    bm[k] = fabs_(sp[k].R.h) * (fabs_(M[k].h * y1.h) + fabs_(be[k].h));
     al[k] = ff_mul(sp[k].R, ff_sub(ff_mul(M[k], y0), al[k]));
     be[k] = ff_mul(sp[k].R, ff_sub(ff_mul(M[k], y1), be[k]));
   }
   // Newton from the mean pressure, in FP32
-  float x = 0.5f * dP.h;
+  float x = 0.5f * dP.h, pm = 3e38f;   // pm: the distance to the nearest pole
   for (int it = 0; it < 8; ++it) {
-    float V = 0.f, dV = 0.f, pm = 3e38f;
+    float V = 0.f, dV = 0.f;
+    pm = 3e38f;
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
       const float q = (P0.h + x) + sp[k].pinf.h;
@@ -112,13 +119,14 @@ MPMC_FF bool face_avg_ff(const SpeciesFF* sp, const double* mi, const double* mj
     x += dx;
     if (!(fabs_(dx) > 1.5e-5f * pm)) break;
   }
-  // two steps in float-float (the derivative in FP32), and the sums at the root
+  // two steps with a float-float residual (derivative and step in FP32), a third
+  // where the second was not yet small (trace gas in a liquid across a jump,
+  // whose FP32 root is off by parts in a thousand), and the sums at the root
   ff xx = {x, 0.f}, s1, s2;
-  float dx = 0.f, pm = 3e38f;
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
+  float dx = 0.f, dV = 0.f;
+  for (int it = 0; it < 3; ++it) {
     ff V = {0.f, 0.f};
-    float dV = 0.f;
+    dV = 0.f;
     const ff p = ff_add(P0, xx);
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -131,10 +139,13 @@ MPMC_FF bool face_avg_ff(const SpeciesFF* sp, const double* mi, const double* mj
     }
     dx = -V.h * frcp(dV);
     xx = ff_add(xx, ff{dx, 0.f});
+    if (it > 0 && !(fabs_(dx) > 1e-10f * pm)) break;
   }
+  pm = 3e38f;
   const ff p = ff_add(P0, xx), T = ff_add(T0, ff_add(y0, ff_mul(y1, xx)));
   s1 = {0.f, 0.f};
   s2 = {0.f, 0.f};
+  float s3 = 0.f, mV = 0.f;
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const ff q = ff_add(p, sp[k].pinf);
@@ -142,13 +153,19 @@ MPMC_FF bool face_avg_ff(const SpeciesFF* sp, const double* mi, const double* mj
     const ff r = M[k].h != 0.f ? ff_rcp(q) : ff{0.f, 0.f};
     const ff t = ff_mul(ff_mul(sp[k].R, M[k]), r);
     s1 = ff_add(s1, t);
-    s2 = ff_add(s2, ff_mul(t, r));
+    const ff tr = ff_mul(t, r);
+    s2 = ff_add(s2, tr);
+    s3 += fabs_(tr.h * r.h);
+    mV += (am[k] + bm[k] * fabs_(xx.h)) * fabs_(r.h);
   }
   const ff Q = ff_mul(T, ff_sub(ff_mul(cpM, s2), ff_sqr(s1)));
+  // what the terms' rounding (2^-46 of their magnitudes) leaves in p, times
+  // d ln c / d p, in 2^-45
+  const float rel = mV * s3 * fabs_(frcp(dV * s2.h));
   const ff Xf = ff_mul(ff_mul(T, s1), inv);
   const ff cf = ff_sqrt(ff_mul(ff_mul(cpM, Mt), ff_rcp(Q)));
   const float LO = 8.67e-19f, HI = 1.15e18f;   // 2^-60, 2^60
-  const bool ok = fabs_(dx) <= 2.4e-7f * pm && pm > LO && pm < HI && T.h > LO && T.h < HI && Mt.h > LO &&
+  const bool ok = rel <= 16.f && fabs_(dx) <= 1e-9f * pm && pm > LO && pm < HI && T.h > LO && T.h < HI && Mt.h > LO &&
                   cf.h > LO && cf.h < HI && fabs_(Xf.h) < HI && s2.h > 1e-30f;
   if (!ok) return false;
   X = ff_double(Xf);
