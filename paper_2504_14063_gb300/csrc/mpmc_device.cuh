@@ -220,10 +220,12 @@ __device__ __forceinline__ double wget(const KParams& P, const double* __restric
 }
 
 // ---------------------------------------------------------------------------
-// 1/x and 1/sqrt(x) by one third-order step from the hardware's approximation
-// (20 bits: 3 and 5 FP64 operations, an error of an ulp, where the IEEE
-// sequences take 6 to 9).  For finite, normal x; others may give NaN where
-// the division gives infinity or zero.
+// 1/x and 1/sqrt(x) from the hardware's approximation of 20 bits by one step of
+// Householder's method of third order (The Numerical Treatment of a Single
+// Nonlinear Equation, 1970): the series of 1/(1 - e) and (1 - e)^(-1/2) in the
+// residual e to e^2, whose next term is below 2^-57.  3 and 5 FP64 operations, an
+// error of an ulp, where the IEEE sequences take 6 to 9.  For finite, normal x;
+// others may give NaN where the division gives infinity or zero.
 __device__ __forceinline__ double drcp(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -237,8 +239,10 @@ __device__ __forceinline__ double drsqrt(double x) {
   const double e = fma(-(x * y), y, 1.0);
   return fma(e * y, fma(e, 0.375, 0.5), y);
 }
-// a / b with r = 1 / b to an ulp: the residual's correction, which rounds as
-// the division does (but for ties within 2^-53 of an ulp, and subnormals)
+// a / b with r = 1 / b to an ulp, by Markstein's correction with the exact
+// residual (Computation of elementary functions on the IBM RISC System/6000
+// processor, IBM J. Res. Dev. 34, 1990): rounds as the division does, but for
+// quotients within 2^-51 of an ulp of a tie, and subnormals
 __device__ __forceinline__ double ddiv(double a, double b, double r) {
   const double q = a * r;
   return fma(fma(-b, q, a), r, q);

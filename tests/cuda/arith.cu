@@ -57,3 +57,33 @@ extern "C" int probe_cells(const mpmc_grid* g, const mpmc_eos* e, const mpmc_mod
   }
   return cudaDeviceSynchronize() != cudaSuccess;
 }
+
+// |x - y| in units of the last place (same sign, finite)
+__device__ unsigned long long ulps(double x, double y) {
+  const long long d = __double_as_longlong(x) - __double_as_longlong(y);
+  return (unsigned long long)(d < 0 ? -d : d);
+}
+// out: largest errors of [0] drcp, [1] qdiv against CUDA's division, in ulps;
+// [2] drsqrt's in 2^-60 of its value; differences from CUDA's division of ddiv
+// [3] with drcp's reciprocal, [4] with a refined one
+__global__ void k_div(const double* __restrict__ a, const double* __restrict__ b, long long n,
+                      unsigned long long* out) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double x = a[i], y = b[i], r = drcp(y);
+  atomicMax(out, ulps(r, 1.0 / y));
+  atomicMax(out + 1, ulps(qdiv(x, y), x / y));
+  // z = 1 / sqrt(w) (1 + d): w z^2 - 1 = 2 d + d^2, w z^2 as p z + q z exactly
+  const double w = fabs(y), z = drsqrt(w), p = __dmul_rn(w, z), q = __fma_rn(w, z, -p);
+  const double d = 0.5 * __fma_rn(q, z, __fma_rn(p, z, -1.0));
+  atomicMax(out + 2, (unsigned long long)ceil(fabs(d) * 0x1p60));
+  if (ulps(ddiv(x, y, r), x / y)) atomicAdd(out + 3, 1ull);
+  const double r2 = fma(fma(-y, r, 1.0), r, r);
+  if (ulps(ddiv(x, y, r2), x / y)) atomicAdd(out + 4, 1ull);
+}
+
+extern "C" int probe_div(const double* a, const double* b, long long n, unsigned long long* out) {
+  if (n <= 0) return 1;
+  k_div<<<(unsigned)((n + 255) / 256), 256>>>(a, b, n, out);
+  return cudaDeviceSynchronize() != cudaSuccess;
+}

@@ -7,7 +7,13 @@ compositions (down to 1e-14 and, for partial densities below float-float's
 range, 1e-30), 3e3 to 3e7 Pa, 200 to 1700 K, from rest to flow whose kinetic
 energy is 1000 times its thermal energy, for one liquid, two liquids and a NASG
 liquid with covolume and reference energy.  Refusals are legitimate and are
-bounded: at low speed, with no species below the range, at most 5 %."""
+bounded: at low speed, with no species below the range, at most 5 %.
+
+Reciprocals, roots and quotients against CUDA's, over 2^-1000 .. 2^1000 and
+mantissas at the ends of the binade: drcp leaves 2^-57 of its series and one
+rounding (at most 1 ulp from the rounded quotient), drsqrt the roundings of its
+residual and of its last step, 2^-53 (1 + 1/2) (at most 200 of 2^-60), qdiv two
+roundings and drcp's (at most 2 ulp), ddiv the division's own result."""
 import ctypes
 import os
 import subprocess
@@ -75,3 +81,27 @@ def test_mixed_inversion_is_fp64_rounded(probe, name, speed, trace):
     assert differ == [0] * 6
     if speed <= 1 and trace <= 14:
         assert taken >= 0.95 * U.shape[1]
+
+
+@pytest.mark.parametrize("kind", ["random", "ends", "near"])
+def test_reciprocals_roots_and_quotients(probe, kind):
+    n = 8_000_000
+    g = torch.Generator("cuda").manual_seed(5)
+    r = lambda: torch.rand(n, generator=g, device="cuda", dtype=torch.float64)
+    if kind == "near":      # ordinary sizes, quotients near one
+        b = 1.0 + r()
+        a = b * (1.0 + 1e-9 * (r() - 0.5))
+    else:
+        m = 1.0 + r()
+        if kind == "ends":  # within 64 ulp of a power of two, on either side
+            m = 1.0 + torch.randint(-64, 65, (n,), generator=g, device="cuda").double() * 2.0 ** -53
+        pow2 = lambda lim: ((torch.randint(-lim, lim, (n,), generator=g, device="cuda") + 1023) << 52).view(torch.float64)
+        b = m * pow2(999)
+        a = (1.0 + r()) * pow2(20)
+        b = torch.where(r() < 0.5, -b, b)
+    out = torch.zeros(8, dtype=torch.int64, device="cuda")
+    assert probe.probe_div(ctypes.c_void_p(a.data_ptr()), ctypes.c_void_p(b.data_ptr()), ctypes.c_longlong(n),
+                           ctypes.c_void_p(out.data_ptr())) == 0
+    rcp, quo, root, d1, d2 = out.cpu().tolist()[:5]
+    print(f"{kind}: drcp {rcp} ulp, qdiv {quo} ulp, drsqrt {root} of 2^-60, ddiv differs {d1} and {d2}")
+    assert rcp <= 1 and quo <= 2 and root <= 200 and d1 == 0 and d2 == 0
