@@ -156,6 +156,18 @@ int pt_equilibrium(const orc_params& p, const R* Y, const R& e, const R& v, R& P
                   ? lo
                   : hi;
     P = R(P0);
+    if (std::is_same<R, long double>::value) {
+      /* from the double root to that of the extended residual: Newton steps */
+      for (it = 0; it < 3; ++it) {
+        R dfdP(0.0);
+        for (int k = 0; k < p.ns; ++k)
+          if (Yv[k] != 0.0) {
+            R den = P + p.pinf[k];
+            dfdP = dfdP - Y[k] * Rgas(p, k) * (Ep - p.pinf[k]) / (den * den);
+          }
+        P = P - pt_residual<R>(p, Y, Ep, Cv, P) / dfdP;
+      }
+    }
     if (is_dual<R>::value) {
       /* derivative of the root by the implicit-function theorem: one Newton
        * step taken in R arithmetic from the converged value */
@@ -1553,6 +1565,20 @@ int orc_stage(const orc_params* p, const double* U_n, const double* U_k, double 
   if (check(p)) return ORC_INVALID;
   Solver<double> s(*p);
   return s.stage(U_n, U_k, rk0, rk1, rk2, dt, Gamma, U_out, dUdt, flags);
+}
+
+int orc_stage_ext(const orc_params* p, const double* U_n, const double* U_k, double rk0, double rk1,
+                  double rk2, double dt, double Gamma, double* dUdt, double* dUdt_lo) {
+  if (check(p)) return ORC_INVALID;
+  Solver<long double> s(*p);
+  const size_t n = (size_t)s.nv * s.G.ncell;
+  std::vector<long double> Un(U_n, U_n + n), Uk(U_k, U_k + n), L(n);
+  int st = s.stage(Un.data(), Uk.data(), rk0, rk1, rk2, dt, (long double)Gamma, nullptr, L.data(), nullptr);
+  for (size_t i = 0; i < n; ++i) {
+    dUdt[i] = (double)L[i];
+    dUdt_lo[i] = (double)(L[i] - (long double)dUdt[i]);
+  }
+  return st;
 }
 
 int orc_face_fluxes(const orc_params* p, const double* U_n, const double* U_k, double rk0,

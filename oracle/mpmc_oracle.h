@@ -141,6 +141,11 @@ int orc_physical_flux(const orc_params* p, int d, const double* W, double* F);
 /* conserved vector of a primitive point state W (layout as in orc_hllc_prim) */
 int orc_cons_from_point(const orc_params* p, const double* W, double* U);
 
+/* dUdt of one stage in long double arithmetic from the double states, as an
+ * unevaluated sum dUdt + dUdt_lo (TENO6's moment matrices stay double) */
+int orc_stage_ext(const orc_params* p, const double* U_n, const double* U_k, double rk0, double rk1,
+                  double rk2, double dt, double Gamma, double* dUdt, double* dUdt_lo);
+
 /* Forward-mode tangents (directional derivatives of the discrete map, its
  * branches taken on values; dt and Gamma frozen), the CPU reference for the
  * discrete adjoint.  Each returns the primal outputs as well. */

@@ -117,6 +117,7 @@ def _declare(L):
         "orc_hllc_prim": [P, i, _dp, _dp, _dp],
         "orc_physical_flux": [P, i, _dp, _dp],
         "orc_cons_from_point": [P, _dp, _dp],
+        "orc_stage_ext": [P, _dp, _dp, d, d, d, d, d, _dp, _dp],
         "orc_stage_jvp": [P, _dp, _dp, _dp, d, d, d, d, d, _dp, _dp],
         "orc_rk_step_jvp": [P, _dp, _dp, d, d, _dp, _dp],
         "orc_primitives_jvp": [P, _dp, _dp, _dp, _dp],
@@ -229,6 +230,13 @@ class Oracle:
         st = self.lib.orc_stage(self.pp, _ptr(U_n), _ptr(U_k), rk[0], rk[1], rk[2], dt, Gamma,
                                 _ptr(Uo), _ptr(L), _ptr(fl))
         return Uo, L, fl, st
+
+    def stage_ext(self, U_n, U_k, rk, dt, Gamma):
+        """dUdt in long double, as (high, low) parts."""
+        U_n, U_k = np.ascontiguousarray(U_n), np.ascontiguousarray(U_k)
+        hi, lo = np.zeros_like(U_k), np.zeros_like(U_k)
+        self.lib.orc_stage_ext(self.pp, _ptr(U_n), _ptr(U_k), rk[0], rk[1], rk[2], dt, Gamma, _ptr(hi), _ptr(lo))
+        return hi, lo
 
     def face_fluxes(self, U_n, U_k, rk=(1.0, 0.0, 1.0), dt=0.0, Gamma=0.0):
         tot = sum(self.nfaces(d) for d in range(self.problem.dim)) * self.nv

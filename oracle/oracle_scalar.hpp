@@ -1,6 +1,7 @@
 /*
  * Scalar helpers of the CPU oracle (test infrastructure only): the plain
- * double type, and a forward-mode dual number Dual<N> carrying N tangent
+ * double type, long double (a right-hand side in extended precision, against
+ * which the errors of FP64 ones are measured), and a forward-mode dual number Dual<N> carrying N tangent
  * directions, so that the oracle's own arithmetic, unchanged, also yields
  * exact directional derivatives (used as the CPU reference gradient for the
  * discrete adjoint).  Branches compare values only.
@@ -19,6 +20,7 @@ using std::sqrt;
 using std::tanh;
 
 inline double val(double x) { return x; }
+inline double val(long double x) { return (double)x; }
 
 template <class R>
 struct is_dual : std::false_type {};
@@ -103,6 +105,7 @@ template <int N> inline Dual<N> fabs(const Dual<N>& a) { return a.v < 0.0 ? -a :
 
 /* x with its value replaced by v and its tangent kept */
 inline double with_value(double, double v) { return v; }
+inline long double with_value(long double, double v) { return v; }
 template <int N> inline Dual<N> with_value(const Dual<N>& x, double v) {
   Dual<N> r = x;
   r.v = v;

@@ -224,7 +224,8 @@ __device__ __forceinline__ bool limit_Y(double* Y, const double* Yc) {
 // liquid is a small difference); several distinct Pinf: the residual's root
 // from FP32, then a float-float Halley step (to ~2^-46 of the residual's
 // terms), then one Newton step whose residual is FP64; the general iteration
-// where that step is not small against the distance to the nearest pole.
+// where that step is above 5e-10 of the distance to the nearest pole (its
+// derivative is FP32: 2^-21 of a step, 2^-52 of that distance at most).
 template <int NS>
 __device__ __forceinline__ int cell_pt(const KParams& P, const double* Y, double e, double v, double& p, double& T,
                                        double* r) {
@@ -335,7 +336,7 @@ __device__ __forceinline__ int cell_pt(const KParams& P, const double* Y, double
       if (nonzero(Y[k])) fd = fma(w[k], r[k], fd);
     }
     const float dxf = -narrow(fd) / df;
-    if (big < (1023 + 100) << 20 && fabsf(dxf) <= 1e-7f * (xx.h - lof) && xx.h < 1e30f) {
+    if (big < (1023 + 100) << 20 && fabsf(dxf) <= 5e-10f * (xx.h - lof) && xx.h < 1e30f) {
       const double dx = ff_widen(dxf, 1023);
       p += dx;
 #pragma unroll
@@ -353,7 +354,7 @@ __device__ __forceinline__ int cell_pt(const KParams& P, const double* Y, double
   for (int k = 0; k < NS; ++k)
     if (nonzero(Y[k])) {
       const double c = Y[k] * P.cv[k];
-      den += nonzero(P.pinf[k]) ? (c * fma(P.gam[k], P.pinf[k], p)) * r[k] : c;
+      den = add_(den, nonzero(P.pinf[k]) ? ddiv(mul_(c, add_(p, mul_(P.gam[k], P.pinf[k]))), p + P.pinf[k], r[k]) : c);
     }
   T = normal_(den) ? ddiv(em, den, drcp(den)) : em / den;
   return st;
@@ -430,38 +431,45 @@ __global__ void __launch_bounds__(CELL_THREADS)
     double mu = 0.0, lam = 0.0;
     if (P.cdi || P.diffusion || P.viscous) {
       double phi[2], Yp[2];
-      const double rT = rho * T;
 #pragma unroll
       for (int ph = 0; ph < 2; ++ph) {
-        // phi_p = sum U_k v_k = rho T sum z_k + sum U_k b_k, h_p rho_p phi_p = sum U_k h_k
-        double f = 0.0, hr = 0.0, yp = 0.0, hb = 0.0, hq = 0.0;
+        // phi_p = sum U_k v_k, h_p rho_p phi_p = sum U_k h_k in the oracle's
+        // order and rounding, the quotients corrected: the regularization flux is
+        // the difference of phi against its sharpening, and with a rounding or two
+        // more in phi the right-hand side's error in a liquid was 1.1 to 1.5 times
+        // as large (bubble, shock onto a droplet)
+        double f = 0.0, hr = 0.0, yp = 0.0;
 #pragma unroll
         for (int k = 0; k < NS; ++k)
           if (P.phase[k] == ph) {
             yp += Y[k];
-            f += z[k];
-            hr = fma(Uc[k], P.cp[k], hr);
-            if (P.has_b) hb = fma(Uc[k], P.b[k], hb);
-            if (P.has_q) hq = fma(Uc[k], P.q[k], hq);
+            if (nonzero(Uc[k])) {
+              double vk = ddiv(mul_(P.Rk[k], T), add_(p, P.pinf[k]), r[k]), hk = mul_(P.cp[k], T);
+              if (P.has_b) {
+                vk = add_(vk, P.b[k]);
+                hk = add_(hk, mul_(P.b[k], p));
+              }
+              if (P.has_q) hk = add_(hk, P.q[k]);
+              f = add_(f, mul_(Uc[k], vk));
+              hr = add_(hr, mul_(Uc[k], hk));
+            }
           }
-        f = fma(rT, f, hb);
-        hr *= T;
-        if (P.has_b) hr = fma(p, hb, hr);
-        if (P.has_q) hr += hq;
         phi[ph] = f;
         Yp[ph] = yp;
         if (P.cdi) {
-          const bool present = yp >= ABSENT;
-          const double rf = qdiv(1.0, f);
-          Wc[(P.wHrho + ph) * ws + c] = present ? hr * rf : 0.0;
+          const bool present = yp >= ABSENT, norm = normal_(f);
+          const double rf = norm ? drcp(f) : 0.0;
+          Wc[(P.wHrho + ph) * ws + c] = present ? (norm ? ddiv(hr, f, rf) : hr / f) : 0.0;
 #pragma unroll
           for (int k = 0; k < NS; ++k)
-            if (P.phase[k] == ph) Wc[(P.wYrho + k) * ws + c] = present ? Uc[k] * rf : 0.0;
+            if (P.phase[k] == ph)
+              Wc[(P.wYrho + k) * ws + c] = present ? (norm ? ddiv(Uc[k], f, rf) : Uc[k] / f) : 0.0;
         }
       }
       if (P.cdi) {
         Wc[P.wPhi0 * ws + c] = phi[0];
-        Wc[P.wPsi * ws + c] = P.cdi_eps * log(qdiv(phi[0] + P.psi_delta, phi[1] + P.psi_delta));
+        const double num = phi[0] + P.psi_delta, den = phi[1] + P.psi_delta;
+        Wc[P.wPsi * ws + c] = P.cdi_eps * log(normal_(den) ? ddiv(num, den, drcp(den)) : num / den);
       }
       // phase viscosities: liquid constant, gas by Wilke's rule
       double mup[2] = {P.mu_liquid, 0.0};
