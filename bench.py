@@ -56,12 +56,12 @@ L2_BYTES = 129 * 2 ** 20
 # and while the kernels' sources hash to the captured version (None
 # otherwise).
 TRAFFIC_GRID = 256
-TRAFFIC = {"k_face": 9.706e9, "mx::k_face": 3.321e9, "k_prim": 4.260e9, "mx::k_prim": 3.190e9,
-           "k_update": 5.993e9, "mx::k_update": 4.294e9}
+TRAFFIC = {"k_face": 9.621e9, "mx::k_face": 3.320e9, "k_prim": 4.246e9, "mx::k_prim": 3.200e9,
+           "k_update": 5.964e9, "mx::k_update": 4.303e9}
 TRAFFIC_SOURCES = tuple("paper_2504_14063_gb300/csrc/" + f for f in (
     "mpmc_kernels.cuh", "mpmc_device.cuh", "mpmc_ff.h", "mpmc_avg.h", "mpmc_fast.cuh", "mpmc_kernels_d3.cu",
     "mpmc_fast_d3.cu", "mpmc_mixed.cuh", "mpmc_mixed_d3.cu", "mpmc_update.cuh"))
-TRAFFIC_SHA256 = "967111c73c4347f68a056f8800f2232316c8c00d8f38ba94677b44d1558ed938"
+TRAFFIC_SHA256 = "d9a68dc50ca7b7d271ccae1ee5801cec5e87d429eaf18375cb80abe42bce1831"
 
 
 def sources_sha256():
@@ -405,21 +405,20 @@ def adjoint_section(mp, torch, nsteps=200, every=20, n=512):
     lam = torch.randn(Ud.shape, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(0))
     lam_n = torch.empty_like(lam)
     Uf = Ud.clone()
-    reps = 5
-    ef = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(reps)]
-    ea = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(reps)]
-    for r in range(reps):
-        Uf.copy_(Ud)
-        ef[r][0].record()
-        ctx.rk_step(Uf, dt)
-        ef[r][1].record()
-    for r in range(reps):
-        ea[r][0].record()
-        ctx.rk_step_adjoint(Ud, lam, dt=dt, tape=tape, lam_n=lam_n, stages=stages)
-        ea[r][1].record()
-    torch.cuda.synchronize()
-    dense_f = float(np.median([x.elapsed_time(y) for x, y in ef]))
-    dense_a = float(np.median([x.elapsed_time(y) for x, y in ea]))
+
+    def median_ms(call, reps=5):
+        ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(reps)]
+        for b, e in ev:
+            Uf.copy_(Ud)
+            b.record()
+            call()
+            e.record()
+        torch.cuda.synchronize()
+        return float(np.median([b.elapsed_time(e) for b, e in ev]))
+
+    dense_f = median_ms(lambda: ctx.rk_step(Uf, dt))
+    dense_r = median_ms(lambda: ctx.rk_step_replay(Uf, dt))
+    dense_a = median_ms(lambda: ctx.rk_step_adjoint(Ud, lam, dt=dt, tape=tape, lam_n=lam_n, stages=stages))
     del Ud, Uf, stages, tape, lam, lam_n
     # forward and backward timed alike, the library's per-launch events off
     a = amps0.clone().requires_grad_(True)
@@ -431,6 +430,16 @@ def adjoint_section(mp, torch, nsteps=200, every=20, n=512):
     e[2].record()
     torch.cuda.synchronize()
     fwd_ms, bwd_ms = e[0].elapsed_time(e[1]), e[1].elapsed_time(e[2])
+    # the same steps without a derivative
+    Uf = ctx.init_state(torch.from_numpy(p.prim))
+    ctx.rk_step(Uf.clone(), dt_ic)
+    e[0].record()
+    for _ in range(nsteps):
+        ctx.rk_step(Uf, dt_ic)
+    e[1].record()
+    torch.cuda.synchronize()
+    plain_ms = e[0].elapsed_time(e[1])
+    del Uf
     # the backward's per-family kernel times from a second rollout with them on
     a2 = amps0.clone().requires_grad_(True)
     _, J2, _ = forward(a2, nsteps)
@@ -447,9 +456,14 @@ def adjoint_section(mp, torch, nsteps=200, every=20, n=512):
                         f"step, {dt_ic:.4e} s), checkpoint every {every} steps",
             "functional": f"sum_k dt_k mean_y P(x={col}, y, t_k); gradient w.r.t. 16 interface Fourier amplitudes",
             "forward_ms": fwd_ms, "backward_ms": bwd_ms, "ratio": bwd_ms / fwd_ms,
-            "dense_step": {"forward_ms": dense_f, "adjoint_ms": dense_a, "ratio": dense_a / dense_f,
-                           "note": "one SSP-RK3 step vs its reverse (stage states and flags recorded) "
-                                   "with a dense random adjoint, median of 5"},
+            "undifferentiated": {"forward_ms": plain_ms, "ratio": bwd_ms / plain_ms,
+                                 "note": "the same steps by rk_step, whose faces run in float-float; the rollout's "
+                                         "forward runs the recording FP64 kernels and records its last segment"},
+            "dense_step": {"forward_ms": dense_f, "replay_ms": dense_r, "adjoint_ms": dense_a,
+                           "ratio": dense_a / dense_f, "ratio_to_replay": dense_a / dense_r,
+                           "note": "one SSP-RK3 step (rk_step; rk_step_replay, in the reverse step's arithmetic) "
+                                   "vs its reverse (stage states and flags recorded) with a dense random adjoint, "
+                                   "median of 5"},
             "backward_kernel_ms": {k: v[0] for k, v in prof.items() if v[1]},
             "timing": "forward and backward each bracketed by CUDA events with the library's per-launch "
                       "events off; backward_kernel_ms from a second rollout with them on",
@@ -747,7 +761,8 @@ def main():
                                 "FP64 flux differences and RK combination; bytes and flops averaged over "
                                 "the three stages"),
         "mx::k_update": hbm("mx::k_update", kpm["update"][0], upd_bm,
-                            "FP32 fluxes, differenced and summed in float-float, RK combination in FP64"),
+                            "FP32 fluxes, their differences summed to FP64 rounding, RK combination in FP64 "
+                            "(FP64 pipe 78 % busy in an ncu capture at 128^3)"),
     }
     roofline["note"] = ("operations of the method as itemized; the interpolation's weights, the face average's "
                         "scalars and the sound speed run in float-float on the FP32 pipe, so that the rate in "
@@ -757,7 +772,7 @@ def main():
     rooflines["k_prim"] = hbm("k_prim", kp["prim"][0], prim_bytes(p, n_w64, 8),
                               "p-T inversion iterated on the FP32 pipe, finished in FP64; " + prim_note)
     rooflines["mx::k_prim"] = hbm("mx::k_prim", kpm["prim"][0], prim_bytes(p, n_w64, 4),
-                                  "float-float p-T inversion, FP32 cache (issue-bound: 63 % of the issue slots, "
+                                  "float-float p-T inversion, FP32 cache (issue-bound: 62 % of the issue slots, "
                                   "FP64 pipe 1 %, in an ncu capture at 128^3); " + prim_note)
     mixed = {"value": vm, "unit": UNIT, "ms_per_step": 1e3 * tm / args.steps, "speedup_vs_fp64": vm / value,
              "clocks": clk_m, "kernel_ms_per_step": {k: v[0] * v[1] for k, v in kpm.items()},

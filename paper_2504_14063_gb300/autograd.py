@@ -200,7 +200,9 @@ def primitives(ctx, U):
 
 def rollout(ctx, U0, n, every=20, probe=None, dt=0.0):
     """dt > 0: every step has that length; otherwise each step takes the CFL
-    step of its own U^k (recorded, and frozen in the backward pass)."""
+    step of its own U^k (recorded, and frozen in the backward pass).  With and
+    without a gradient it takes the same steps, in the arithmetic that the
+    backward pass linearizes; ctx.step_n rounds otherwise and is faster."""
     if ctx.precision != _b.FP64:
         raise ValueError("the discrete adjoint needs an FP64 context")
     grad = torch.is_grad_enabled() and U0.requires_grad

@@ -78,7 +78,7 @@ struct KParams {
   SpeciesFF sff[MAXS];       // Rk, cv, cp, pinf as float-floats
   double iW[MAXS], WSc[MAXS];  // 1 / W, W / Sc
   double inv_cdi_eps;        // 1 / cdi_eps
-  double cdi_eps_dx, gtol2;  // 1 / cdi_eps, cdi_eps / dx, (4 GTOL dx)^2
+  double cdi_eps_dx, gtol2;  // cdi_eps / dx, (4 GTOL dx)^2
 };
 
 // fills P.f32 from the FP64 fields (host)

@@ -1,12 +1,14 @@
 // The forward FP64 face pass (arXiv 2504.14063): mpmc_kernels.cuh's k_face
 // with the parts of its arithmetic that act on the cells' differences only
 // moved from the FP64 pipe (2 operations per clock and SM on GB300) to
-// float-float on the FP32 pipe (mpmc_ff.h says what that rests on).  The
-// FP64 pipe bounds the pass (86 % busy); WENO5-Z was half of its operations.
-// Face passes of one SSP-RK3 step with all interpolation in FP64 and so:
-// shock-bubble 1024 x 512 8.70 -> 5.44 ms, droplet field 128^3 79.7 -> 54.2 ms.
-// The right-hand sides' error against extended precision went from 1 to
-// 0.5 .. 1.1 of the FP64 form's (four workloads, every field).
+// float-float on the FP32 pipe (mpmc_ff.h says what that rests on).  Face
+// passes of one SSP-RK3 step, all FP64 and so: shock-bubble 1024 x 512 8.70 ->
+// 2.88 ms, droplet field 128^3 79.7 -> 26.0 ms.  Of the plain form's FP64
+// instructions about 590 per face are left (3D, four species, CDI and diffusion);
+// the pipe is 70 % busy with them (86 % before) at 25 % of the warps, the rest
+// latency of the FP32 chains and of instruction fetches.
+// The right-hand sides' error against extended precision is 0.5 to 1.0 of the
+// FP64 form's (four workloads, every field; tests/test_gpu_forward_accuracy.py).
 //
 // Steps and right-hand sides run these kernels, unless they return limiter
 // flags for a reverse pass.  Those, the recording calls of the discrete adjoint
@@ -1089,7 +1091,8 @@ struct FaceImpl {
     if constexpr (D < 3) {
       // up to two split blocks per SM; with more the redundant X and c cost more
       // than the shorter chain gives (TENO6 faces of 322 x 51 cells: 130 us whole,
-      // 274 us split; 5996 cells: 58 whole, 56 split)
+      // 274 us split; 5996 cells: 58 whole, 56 split).  3D grids in use have more
+      // faces than that (24^3 cells: 14,400); the form is not built for them.
       if (nf <= 2 * 152 * 32) {
         constexpr int nt = 32 * SPLIT_WARPS<NS, D>;
         if (d == 0)

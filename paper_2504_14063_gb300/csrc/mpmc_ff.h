@@ -1,5 +1,6 @@
 // Float-float arithmetic (an unevaluated sum h + l of two FP32 numbers, about
-// 48 significant bits) and the WENO5-Z interpolation on it.
+// 48 significant bits) and the ENO-type interpolations on it (WENO5-Z, WENO5-JS,
+// TENO5, TENO6).
 //
 // Why: one SM of GB300 retires two FP64 operations per clock and 128 FP32
 // ones, so an FP64 instruction costs the time of 64 FP32 instructions, while
@@ -123,7 +124,7 @@ MPMC_FF double dfma(double a, double b, double c) {
 MPMC_FF int imax(int a, int b) { return a > b ? a : b; }
 MPMC_FF int imin(int a, int b) { return a < b ? a : b; }
 
-// |a| >= |b| assumed: the sum and its rounding error
+// |a| >= |b| assumed: the sum and its rounding error (Dekker)
 MPMC_FF ff ff_fast(float a, float b) {
   const float s = fadd(a, b);
   return {s, fadd(b, -fadd(s, -a))};

@@ -1285,12 +1285,13 @@ __global__ void __launch_bounds__(FACE_THREADS, 5)
   }
 }
 
-// divergence of the FP32 fluxes (their differences in float-float) and RK
-// combination in FP64.  Bound by the latency of its 64 loads per cell (3D, four
-// species): three blocks per SM (80 registers) keep most of a cell's loads in
-// flight; one (104 registers) left too few warps, four (64) too few loads per
-// warp.  256^3, per step of three: 5.8 (unbounded), 3.5 (three), 4.6 ms (four);
-// 1.2 ms per launch are 3.7 TB/s of the 267 bytes per cell it must move.
+// divergence of the FP32 fluxes (ff_diff_sum) and RK combination in FP64.  The
+// FP64 pipe bounds it (78 % busy: 43 instructions per cell, 3D, four species)
+// together with the latency of its 64 loads per cell: three blocks per SM (80
+// registers) keep most of them in flight; one (104 registers) left too few warps,
+// four (64) too few loads per warp (256^3, per step of three, with one FP64
+// addition per component fewer: 5.8 unbounded, 3.5 three, 4.6 ms four; now 4.3).
+// 1.4 ms per launch are 3.2 TB/s of the 267 bytes per cell it must move.
 template <int NS, int D>
 __global__ void __launch_bounds__(CELL_THREADS, 3)
     k_update(const KParams P, const double* __restrict__ Un, const double* __restrict__ Uk,
