@@ -91,3 +91,29 @@ def test_backward_of_a_rollout_holds_one_segment(mods, monkeypatch, n, every, ke
     rest = 12 * state
     assert peak <= (0 if kept and n % every == 0 else one) + rest
     assert rest < 0.5 * one
+
+
+def test_reverse_step_under_capture_allocates_nothing(mods):
+    """A reverse step captured before the second cache exists takes the route
+    without it, bit for bit the same."""
+    _, mp = mods
+    p = W.random_smooth_2d(nx=61, ny=47, seed=3)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ctx = mp.Context(p, stream=s)
+        U0 = ctx.init_state(torch.from_numpy(p.prim))
+        lam = torch.randn(U0.shape, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(0))
+        dt = 0.5 * float(ctx.dt_gamma(U0)[0])
+        out, ref = torch.empty_like(U0), torch.empty_like(U0)
+        ctx.rhs_adjoint(U0, None, None, lam, torch.zeros_like(U0))   # the scratch, without the second cache
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        ctx.rk_step_adjoint(U0, lam, dt, None, out)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        ctx.rk_step_adjoint(U0, lam, dt, None, ref)
+    s.synchronize()
+    assert float(ref.abs().max()) > 0 and torch.equal(out, ref)
