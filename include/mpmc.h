@@ -193,7 +193,7 @@ int mpmc_init_state(mpmc_ctx* ctx, const double* prim, double* U);
  * 1, then 2, each laid out like cells with n[d]+1 entries along d.  With
  * flags the call runs in the arithmetic that mpmc_rhs_adjoint recomputes in
  * (dUdt, dt and Gamma then differ from the call's without flags by rounding,
- * and it takes about twice as long). */
+ * and it takes two to three times as long). */
 int mpmc_rhs(mpmc_ctx* ctx, const double* U, double* dUdt, const mpmc_stage* stage, uint32_t* flags);
 
 /* One SSP-RK3 step (Eq. SSPRK3) in place on device array U.  dt > 0: fixed
